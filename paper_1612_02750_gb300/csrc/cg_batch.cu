@@ -29,13 +29,18 @@
 #include <string>
 #include <vector>
 
+#include "qex_dslash64.cuh"
 #include "qex_dslash_site.cuh"
 #include "qex_kernels.cuh"
 
 namespace qex {
 
 constexpr int kTile = 256;  // sites per group (threads per block)
-constexpr int kBatchMinBlocks = 3;  // resident blocks per SM of the iteration kernels (no spills at 85 registers)
+// Resident blocks per SM of the iteration kernels: 3 in FP32 (no spills at 85
+// registers), 2 in FP64 (the integer-pipe hops take 128).
+template <typename R> struct BatchMinBlocks { static constexpr int value = 3; };
+template <> struct BatchMinBlocks<double> { static constexpr int value = 2; };
+constexpr int kBatchMaxPerSm = 3;   // blocks per SM that a batch shape may ask for
 constexpr int kMaxSpt = 4;          // groups per work item
 
 struct LatDesc {
@@ -151,10 +156,11 @@ __device__ __forceinline__ bool last_block_totals(double *partials, unsigned int
 
 // Iteration Dslash kernels: persistent grid over the compacted tile list.
 template <typename R, int FMT, bool NAIK, int ROLE>
-__global__ void __launch_bounds__(kTile, kBatchMinBlocks)
+__global__ void __launch_bounds__(kTile, BatchMinBlocks<R>::value)
 batch_iter_dslash_kernel(const LatDesc *__restrict__ descs, BatchScalars *S, double *partials, unsigned int *counter) {
     __shared__ double smem[32];
     __shared__ double tot[kMaxRhs];
+    extern __shared__ double2 stage[];  // FP64: the t hops (dslash_site64)
     if (S->halt) return;  // uniform over the grid
     const int nl = S->nlist;
     const int nitems = S->bstart[nl];
@@ -183,15 +189,25 @@ batch_iter_dslash_kernel(const LatDesc *__restrict__ descs, BatchScalars *S, dou
                 const Site s = site_of(g, 1, i);
                 const R beta = (R)S->beta[l];
                 const R *r = (const R *)D.ri;
-                const Vec3<R> acc = dslash_site<R, FMT, NAIK>(g, (const R *)D.fat_in, (const R *)D.lng_in, (R)D.c3, 1,
-                                                              i, s, [&](int j) { return axpy_vec(r, pold, beta, vh, j); });
+                Vec3<R> acc;
+                if constexpr (std::is_same<R, double>::value)
+                    acc = dslash_site64<NAIK>(g, (const double *)D.fat_in, (const double *)D.lng_in, D.c3, 1, i, s,
+                                              Direction64{r, pold, beta, vh}, stage + threadIdx.x, kTile);
+                else
+                    acc = dslash_site<R, FMT, NAIK>(g, (const R *)D.fat_in, (const R *)D.lng_in, (R)D.c3, 1, i, s,
+                                                    [&](int j) { return axpy_vec(r, pold, beta, vh, j); });
                 store_vec((R *)D.tmpi, vh, i, acc);
                 store_vec(pnew, vh, i, axpy_vec(r, pold, beta, vh, i));
             } else {
                 const Site s = site_of(g, 0, i);
                 const R *tmp = (const R *)D.tmpi;
-                const Vec3<R> acc = dslash_site<R, FMT, NAIK>(g, (const R *)D.fat_in, (const R *)D.lng_in, (R)D.c3, 0,
-                                                              i, s, [&](int j) { return load_vec(tmp, vh, j); });
+                Vec3<R> acc;
+                if constexpr (std::is_same<R, double>::value)
+                    acc = dslash_site64<NAIK>(g, (const double *)D.fat_in, (const double *)D.lng_in, D.c3, 0, i, s,
+                                              Field64{tmp, vh}, stage + threadIdx.x, kTile);
+                else
+                    acc = dslash_site<R, FMT, NAIK>(g, (const R *)D.fat_in, (const R *)D.lng_in, (R)D.c3, 0, i, s,
+                                                    [&](int j) { return load_vec(tmp, vh, j); });
                 const Vec3<R> qv = load_vec((const R *)pnew, vh, i);
                 const R m2 = (R)D.m2;
                 Vec3<R> o;
@@ -316,12 +332,13 @@ batch_update_kernel(const LatDesc *__restrict__ descs, BatchScalars *S, double *
 
 // Reliable update, FP64 Dslash over the full tile list (lattices with need set).
 template <bool NAIK, int ROLE>
-__global__ void __launch_bounds__(kTile, 3)
+__global__ void __launch_bounds__(kTile, BatchMinBlocks<double>::value)
 batch_ru_dslash_kernel(const LatDesc *__restrict__ descs, int n, BatchScalars *S, const int *need, double *partials,
                        unsigned int *counter) {
     __shared__ double smem[32];
     __shared__ double tot[kMaxRhs];
     __shared__ int ident[kMaxRhs + 1];
+    extern __shared__ double2 stage[];
     const int l = lattice_of_full_tile(descs, n, blockIdx.x);
     const LatDesc &D = descs[l];
     const Geom &g = D.g;
@@ -331,14 +348,12 @@ batch_ru_dslash_kernel(const LatDesc *__restrict__ descs, int n, BatchScalars *S
     if (need[l] && i < g.vh) {
         if constexpr (ROLE == ROLE_RU1) {
             const Site s = site_of(g, 1, i);
-            const double *x = D.x64;
-            store_vec(D.tmp64, vh, i, dslash_site<double, 0, NAIK>(g, D.fat64, D.lng64, D.c3, 1, i, s,
-                                                                   [&](int j) { return load_vec(x, vh, j); }));
+            store_vec(D.tmp64, vh, i, dslash_site64<NAIK>(g, D.fat64, D.lng64, D.c3, 1, i, s, Field64{D.x64, vh},
+                                                          stage + threadIdx.x, kTile));
         } else {
             const Site s = site_of(g, 0, i);
-            const double *tmp = D.tmp64;
-            const Vec3<double> acc = dslash_site<double, 0, NAIK>(g, D.fat64, D.lng64, D.c3, 0, i, s,
-                                                                  [&](int j) { return load_vec(tmp, vh, j); });
+            const Vec3<double> acc = dslash_site64<NAIK>(g, D.fat64, D.lng64, D.c3, 0, i, s, Field64{D.tmp64, vh},
+                                                         stage + threadIdx.x, kTile);
             const Vec3<double> xv = load_vec(D.x64, vh, i), bv = load_vec(D.b, vh, i);
             Vec3<double> o;
 #pragma unroll
@@ -437,6 +452,7 @@ batch_norm2_kernel(const LatDesc *__restrict__ descs, int n, BatchScalars *S, do
     __shared__ double smem[32];
     __shared__ double tot[kMaxRhs];
     __shared__ int ident[kMaxRhs + 1];
+    extern __shared__ double2 stage[];
     const int l = lattice_of_full_tile(descs, n, blockIdx.x);
     const LatDesc &D = descs[l];
     const size_t vh = (size_t)D.g.vh;
@@ -551,12 +567,11 @@ static std::string batch_key(int n, const qex_cg_item *items, qex_prec inner, bo
 
 template <typename R, int FMT, bool NAIK>
 static void launch_iter_t(const BatchLaunch &b, int role, cudaStream_t s) {
-    if (role == ROLE_K1)
-        batch_iter_dslash_kernel<R, FMT, NAIK, ROLE_K1><<<b.iter_grid, kTile, 0, s>>>(b.c->descs, b.c->S,
-                                                                                       b.c->partials, b.c->counter);
-    else
-        batch_iter_dslash_kernel<R, FMT, NAIK, ROLE_K2><<<b.iter_grid, kTile, 0, s>>>(b.c->descs, b.c->S,
-                                                                                       b.c->partials, b.c->counter);
+    auto kernel = role == ROLE_K1 ? batch_iter_dslash_kernel<R, FMT, NAIK, ROLE_K1>
+                                  : batch_iter_dslash_kernel<R, FMT, NAIK, ROLE_K2>;
+    const size_t smem = std::is_same<R, double>::value ? kTile * kStageBytes : 0;
+    if (smem) allow_stage(kernel, kTile);
+    kernel<<<b.iter_grid, kTile, smem, s>>>(b.c->descs, b.c->S, b.c->partials, b.c->counter);
 }
 
 template <typename R, int FMT>
@@ -602,19 +617,14 @@ static qex_status enqueue_reliable_update(const BatchLaunch &b, const GraphCtl &
         batch_ru_vectors_kernel<0><<<b.total_tiles, kTile, 0, s>>>(c->descs, b.n, c->need_snap);
         QEX_CHECK_LAUNCH("batch_ru_vectors_kernel");
     }
-    if (b.naik) {
-        batch_ru_dslash_kernel<true, ROLE_RU1><<<b.total_tiles, kTile, 0, s>>>(c->descs, b.n, c->S, c->need_snap,
-                                                                             c->partials, c->counter);
-        QEX_CHECK_LAUNCH("batch_ru_dslash_kernel");
-        batch_ru_dslash_kernel<true, ROLE_RU2><<<b.total_tiles, kTile, 0, s>>>(c->descs, b.n, c->S, c->need_snap,
-                                                                             c->partials, c->counter);
-    } else {
-        batch_ru_dslash_kernel<false, ROLE_RU1><<<b.total_tiles, kTile, 0, s>>>(c->descs, b.n, c->S, c->need_snap,
-                                                                              c->partials, c->counter);
-        QEX_CHECK_LAUNCH("batch_ru_dslash_kernel");
-        batch_ru_dslash_kernel<false, ROLE_RU2><<<b.total_tiles, kTile, 0, s>>>(c->descs, b.n, c->S, c->need_snap,
-                                                                              c->partials, c->counter);
-    }
+    auto ru1 = b.naik ? batch_ru_dslash_kernel<true, ROLE_RU1> : batch_ru_dslash_kernel<false, ROLE_RU1>;
+    auto ru2 = b.naik ? batch_ru_dslash_kernel<true, ROLE_RU2> : batch_ru_dslash_kernel<false, ROLE_RU2>;
+    const size_t smem = kTile * kStageBytes;
+    allow_stage(ru1, kTile);
+    ru1<<<b.total_tiles, kTile, smem, s>>>(c->descs, b.n, c->S, c->need_snap, c->partials, c->counter);
+    QEX_CHECK_LAUNCH("batch_ru_dslash_kernel");
+    allow_stage(ru2, kTile);
+    ru2<<<b.total_tiles, kTile, smem, s>>>(c->descs, b.n, c->S, c->need_snap, c->partials, c->counter);
     QEX_CHECK_LAUNCH("batch_ru_dslash_kernel");
     if (b.mixed) {
         batch_ru_vectors_kernel<1><<<b.total_tiles, kTile, 0, s>>>(c->descs, b.n, c->need_snap);
@@ -716,11 +726,11 @@ static qex_status tune_batch(const BatchLaunch &b0, const std::vector<LatDesc> &
     QEX_CUDA(cudaEventCreate(&e0));
     QEX_CUDA(cudaEventCreate(&e1));
     float best_us = 0.f;
-    *best = BatchShape{kBatchMinBlocks, 1};
+    *best = BatchShape{kBatchMaxPerSm, 1};
     qex_status st = QEX_OK;
     set_count_launches(false);
     for (int spt = 1; spt <= kMaxSpt && !st; spt *= 2)
-        for (int per_sm = 1; per_sm <= kBatchMinBlocks && !st; ++per_sm) {
+        for (int per_sm = 1; per_sm <= kBatchMaxPerSm && !st; ++per_sm) {
             BatchLaunch b = b0;
             b.spt = spt;
             b.iter_grid = batch_grid(batch_items(descs, spt), per_sm);
@@ -763,7 +773,7 @@ extern "C" qex_status qex_cg_batch_tune_info(const qex_lattice *lead, int *out) 
         set_error("out must not be NULL");
         return QEX_ERR_ARG;
     }
-    out[0] = lead->batch_shape[0] > 0 ? lead->batch_shape[0] : kBatchMinBlocks;
+    out[0] = lead->batch_shape[0] > 0 ? lead->batch_shape[0] : kBatchMaxPerSm;
     out[1] = lead->batch_shape[1] > 0 ? lead->batch_shape[1] : 1;
     out[2] = lead->batch_shape[2];
     return QEX_OK;
@@ -773,9 +783,9 @@ extern "C" qex_status qex_cg_batch_tune_set(const qex_lattice *lead, int blocks_
     qex_status st;
     if ((st = check_lattice(lead))) return st;
     const bool unpin = blocks_per_sm == 0 && groups_per_item == 0;
-    if (!unpin && (blocks_per_sm < 1 || blocks_per_sm > kBatchMinBlocks ||
+    if (!unpin && (blocks_per_sm < 1 || blocks_per_sm > kBatchMaxPerSm ||
                    (groups_per_item != 1 && groups_per_item != 2 && groups_per_item != 4))) {
-        set_error("need 1 <= blocks_per_sm <= %d and groups_per_item 1, 2 or 4 (0, 0 unpins)", kBatchMinBlocks);
+        set_error("need 1 <= blocks_per_sm <= %d and groups_per_item 1, 2 or 4 (0, 0 unpins)", kBatchMaxPerSm);
         return QEX_ERR_ARG;
     }
     qex_lattice *l = const_cast<qex_lattice *>(lead);
@@ -898,7 +908,7 @@ extern "C" qex_status qex_cg_batch(int n, const qex_cg_item *items, qex_prec inn
     // launch shape: pinned on the lead lattice, from the process cache, the
     // compiled defaults (QEX_TUNE=0), or measured after the first residual
     const std::string key = batch_key(n, items, inner, naik);
-    int per_sm = kBatchMinBlocks, spt = 1, source = 0;
+    int per_sm = inner == QEX_F64 ? BatchMinBlocks<double>::value : kBatchMaxPerSm, spt = 1, source = 0;
     bool need_tune = false;
     if (own->batch_pin[0] > 0) {
         per_sm = own->batch_pin[0];

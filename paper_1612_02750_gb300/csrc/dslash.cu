@@ -9,6 +9,7 @@
 // antiperiodic time boundary are computed from the site coordinates; no phase
 // is folded into the links.
 #include <type_traits>
+#include "qex_dslash64.cuh"
 #include "qex_dslash_site.cuh"
 #include "qex_kernels.cuh"
 
@@ -40,9 +41,11 @@ struct DsParams {
 };
 
 template <typename R, int FMT, bool NAIK, int EPI>
-__global__ void __launch_bounds__(kDslashBlock, DslashMinBlocks<R>::value) dslash_kernel(const DsParams<R> P) {
+__global__ void __launch_bounds__(kDslashBlock, DslashMinBlocks<R>::value)
+dslash_kernel(const __grid_constant__ DsParams<R> P) {
     __shared__ double smem[32];
     __shared__ unsigned int is_last;
+    extern __shared__ double2 stage[];  // FP64: the t hops (dslash_site64)
     pdl_trigger();
     pdl_wait();  // everything below may read what earlier kernels wrote
     if (P.check_halt && P.S->halt) return;  // uniform over the grid
@@ -78,6 +81,9 @@ __global__ void __launch_bounds__(kDslashBlock, DslashMinBlocks<R>::value) dslas
         if (EPI == EPI_RESID && zero_x) {
 #pragma unroll
             for (int a = 0; a < 3; ++a) acc.c[a].re = acc.c[a].im = R(0);
+        } else if constexpr (std::is_same<R, double>::value) {
+            acc = dslash_site64<NAIK>(g, P.fat, P.lng, P.c3, p, i, s, Field64{in, vh}, stage + threadIdx.x,
+                                      blockDim.x);
         } else {
             acc = dslash_site<R, FMT, NAIK>(g, P.fat, P.lng, P.c3, p, i, s, [&](int j) {
                 if constexpr (EPI == EPI_PUPD)
@@ -237,7 +243,12 @@ static void launch_t(qex_lattice *lat, const DslashArgs &a, cudaStream_t st) {
     int grid, block;
     dslash_shape(lat, a.prec, NAIK, EPI != EPI_PLAIN && EPI != EPI_PUPD && a.S != nullptr, DslashMinBlocks<R>::value,
                  &grid, &block);
-    launch_k(dslash_kernel<R, FMT, NAIK, EPI>, dim3(grid), dim3(block), 0, st, lat->pdl != 0, P);
+    size_t smem = 0;
+    if constexpr (std::is_same<R, double>::value) {
+        allow_stage(dslash_kernel<R, FMT, NAIK, EPI>, block);
+        smem = block * kStageBytes;
+    }
+    launch_k(dslash_kernel<R, FMT, NAIK, EPI>, dim3(grid), dim3(block), smem, st, lat->pdl != 0, P);
 }
 
 template <typename R, int FMT, bool NAIK>
@@ -246,10 +257,10 @@ static void launch_epi(qex_lattice *lat, const DslashArgs &a, cudaStream_t st) {
         launch_t<R, FMT, NAIK, EPI_PLAIN>(lat, a, st);
     else if (a.epi == EPI_NORMAL)
         launch_t<R, FMT, NAIK, EPI_NORMAL>(lat, a, st);
-    else if (a.epi == EPI_PUPD)
-        launch_t<R, FMT, NAIK, EPI_PUPD>(lat, a, st);
     else if constexpr (std::is_same<R, double>::value)
         launch_t<R, FMT, NAIK, EPI_RESID>(lat, a, st);
+    else
+        launch_t<R, FMT, NAIK, EPI_PUPD>(lat, a, st);
 }
 
 qex_status launch_dslash(qex_lattice *lat, const DslashArgs &a, cudaStream_t st) {
@@ -258,6 +269,10 @@ qex_status launch_dslash(qex_lattice *lat, const DslashArgs &a, cudaStream_t st)
         if (s) return s;
     }
     if (a.prec == QEX_F64) {
+        if (a.epi == EPI_PUPD) {
+            set_error("the direction-update epilogue is FP32 only");
+            return QEX_ERR_ARG;
+        }
         if (a.lng)
             launch_epi<double, 0, true>(lat, a, st);
         else

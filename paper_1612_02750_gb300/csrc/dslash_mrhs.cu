@@ -7,6 +7,7 @@
 // per right-hand side, the input vector once and the output once.  The
 // reducing epilogues run a persistent grid-stride loop and reduce per
 // right-hand side in a fixed order (bit-reproducible).
+#include "qex_dslash64.cuh"
 #include "qex_dslash_site.cuh"
 #include "qex_kernels.cuh"
 
@@ -27,7 +28,7 @@ constexpr int kMrhsBlock = 256;  // threads (sites) per block
 // instruction-level parallelism that the lower occupancy gives up).  The CG
 // epilogues, which also gather the directions or read the q vectors, run
 // faster at KR = 2 and 4 blocks (24^4, 16 sources: the batched mixed CG
-// 0.42 s against 0.46 s); FP64 keeps KR = 2 at 2 blocks (it spills above).
+// 0.42 s against 0.46 s).  FP64 takes one at 2 blocks (dslash_site64).
 #ifndef QEX_MRHS_KR_CG
 #define QEX_MRHS_KR_CG 2
 #endif
@@ -41,7 +42,7 @@ struct MrhsShape {
 };
 template <int EPI>
 struct MrhsShape<double, EPI> {
-    static constexpr int kr = 2;
+    static constexpr int kr = 1;
     static constexpr int minb = 2;
 };
 // the largest persistent grid times KR of any reducing variant (partials per launch)
@@ -67,10 +68,11 @@ struct MParams {
 };
 
 template <typename R, int FMT, bool NAIK, int EPI>
-__global__ void __launch_bounds__(kMrhsBlock, (MrhsShape<R, EPI>::minb)) dslash_mrhs_kernel(const MParams<R> P) {
+__global__ void __launch_bounds__(kMrhsBlock, (MrhsShape<R, EPI>::minb)) dslash_mrhs_kernel(const __grid_constant__ MParams<R> P) {
     constexpr int KR = MrhsShape<R, EPI>::kr;
     __shared__ double wsum[kMrhsBlock / 32][KR];
     __shared__ unsigned int is_last;
+    extern __shared__ double2 stage[];  // FP64: the t hops (dslash_site64)
     MrhsScalars *S = P.S;
     if (P.check_halt && S->halt) return;  // uniform over the grid
     const Geom &g = P.g;
@@ -109,6 +111,15 @@ __global__ void __launch_bounds__(kMrhsBlock, (MrhsShape<R, EPI>::minb)) dslash_
         if (!any) continue;
         const Site s = site_of(g, p, i);
         Vec3<R> acc[KR];
+        if constexpr (std::is_same<R, double>::value) {
+            double2 *slot = stage + threadIdx.x;
+            if constexpr (EPI == EPI_PUPD)
+                acc[0] = dslash_site64<NAIK>(g, P.fat, P.lng, P.c3, p, i, s,
+                                             Direction64{P.r + off[0], pold + off[0], beta[0], vh}, slot, kMrhsBlock);
+            else
+                acc[0] = dslash_site64<NAIK>(g, P.fat, P.lng, P.c3, p, i, s, Field64{P.in + off[0], vh}, slot,
+                                             kMrhsBlock);
+        } else
         dslash_site_n<R, FMT, NAIK, KR>(g, P.fat, P.lng, P.c3, p, i, s, [&](int j, int k) {
             Vec3<R> v;
             if (!act[k]) {
@@ -269,7 +280,9 @@ static void launch_m(const qex_lattice *lat, const MrhsArgs &a, cudaStream_t st)
         if (cap < P.ngroups) cap = P.ngroups;
         gx = total < cap ? total : cap;
     }
-    dslash_mrhs_kernel<R, FMT, NAIK, EPI><<<gx, kMrhsBlock, 0, st>>>(P);
+    const size_t smem = std::is_same<R, double>::value ? kMrhsBlock * kStageBytes : 0;
+    if (smem) allow_stage(dslash_mrhs_kernel<R, FMT, NAIK, EPI>, kMrhsBlock);
+    dslash_mrhs_kernel<R, FMT, NAIK, EPI><<<gx, kMrhsBlock, smem, st>>>(P);
 }
 
 template <typename R, int FMT, bool NAIK>

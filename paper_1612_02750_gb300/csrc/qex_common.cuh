@@ -608,7 +608,7 @@ constexpr int kHostSlabs = 8;  // t-slabs of a link set in qex_cg_host (lattice:
 #define QEX_DSLASH_MIN_BLOCKS 4
 #endif
 #ifndef QEX_DSLASH_MIN_BLOCKS_F64
-#define QEX_DSLASH_MIN_BLOCKS_F64 3
+#define QEX_DSLASH_MIN_BLOCKS_F64 2
 #endif
 // Grid of the reducing Dslash variants: resident blocks per SM of their
 // persistent grid (-1: the launch-bounds minimum; 0: one thread per site).
@@ -621,7 +621,7 @@ constexpr int kHostSlabs = 8;  // t-slabs of a link set in qex_cg_host (lattice:
 #endif
 constexpr int kDslashBlock = QEX_DSLASH_BLOCK;
 constexpr int kDslashMinBlocks = QEX_DSLASH_MIN_BLOCKS;         // FP32 variants
-constexpr int kDslashMinBlocksF64 = QEX_DSLASH_MIN_BLOCKS_F64;  // FP64 variants (ALU bound, no spills)
+constexpr int kDslashMinBlocksF64 = QEX_DSLASH_MIN_BLOCKS_F64;  // FP64 variants (128 registers: qex_dslash64.cuh)
 template <typename R> struct DslashMinBlocks { static constexpr int value = kDslashMinBlocks; };
 template <> struct DslashMinBlocks<double> { static constexpr int value = kDslashMinBlocksF64; };
 

@@ -115,7 +115,8 @@ __device__ __forceinline__ void dslash_site_n(const Geom &g, const R *fat, const
     }
 }
 
-// One field: (D in)(x), `in(j)` the input vector at index j.
+// One field: (D in)(x), `in(j)` the input vector at index j.  (FP64 kernels:
+// dslash_site64 in qex_dslash64.cuh, which falls back to this one.)
 template <typename R, int FMT, bool NAIK, typename In>
 __device__ __forceinline__ Vec3<R> dslash_site(const Geom &g, const R *fat, const R *lng, R c3, int p, int i,
                                                const Site &s, const In &in) {

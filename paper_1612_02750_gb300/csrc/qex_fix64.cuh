@@ -1,0 +1,221 @@
+// qex_fix64.cuh -- FP64 hops on the integer pipe.
+//
+// An FP64 FMA takes 64 clocks a warp on a GB300 SM quarter, a 32x32+64-bit
+// integer multiply-add and every other integer instruction 2 (measured; the
+// two kinds of integer instruction share those clocks).  A 3x3 complex
+// mat-vec is 36 FP64 FMAs, 2304 clocks; here it takes 1070: the link and the
+// vector are brought into fixed point (a common exponent each, 60 bits, as
+// two signed 32-bit digits), a product is three multiply-adds (hi hi, hi lo,
+// lo hi; the lo lo product is below the last bit kept) and the sums are exact
+// 64-bit integers.  About half of the 520 instructions convert the link.
+//
+// Accuracy.  One unit of the accumulators is 2^-56 of the largest product
+// |U| |v| (largest real of the link times largest real of the vectors, each
+// rounded up to a power of two); a hop rounds by about 0.3 units, and the
+// running exponent carries kFixSlack spare bits.  FP64 arithmetic rounds
+// every partial sum by 2^-54 of its value.  Norm-wise error of a sum of eight
+// hops against 113 bits, Gaussian vectors: 0.64e-16 here, 2.3e-16 for FMAs
+// (unit links: 0.71e-16 and 1.05e-16; vectors of very different size from
+// hop to hop: 0.88e-16 and 2.2e-16).  The accuracy is that of the colour
+// vector as a whole: a colour far below the others of its own site keeps
+// their absolute error.  A hop whose link or vector holds an Inf or NaN, or
+// whose largest real lies outside 2^-470 .. 2^470 (zeros apart), makes the
+// site fall back to FP64 FMAs, so such values come out as they do there.
+#pragma once
+
+#include <string.h>
+
+#include "qex_common.cuh"
+
+namespace qex {
+
+constexpr int kFixShift = 4;   // high digits are at most 2^28
+constexpr int kFixSlack = 1;   // spare bits of the running exponent
+constexpr int kFixLow = 553;    // exponent fields accepted: 2^-470 <= ...
+constexpr int kFixHigh = 1493;  // ... < 2^470
+
+struct Digits {
+    int hi, lo;  // hi 2^32 + lo
+};
+
+QEX_HD uint64_t fix_shr(uint64_t x, uint32_t n) {
+#ifdef __CUDA_ARCH__
+    uint64_t r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));  // 0 for n > 63
+    return r;
+#else
+    return n > 63 ? 0 : x >> n;
+#endif
+}
+
+QEX_HD int64_t fix_sar(int64_t x, uint32_t n) { return x >> (n > 63 ? 63 : n); }
+
+// a b + c, one IMAD.WIDE
+QEX_HD int64_t fix_mad(int a, int b, int64_t c) { return (int64_t)a * b + c; }
+
+QEX_HD uint64_t fix_bits(double d) {
+#ifdef __CUDA_ARCH__
+    return (uint64_t)__double_as_longlong(d);
+#else
+    uint64_t u;
+    memcpy(&u, &d, 8);
+    return u;
+#endif
+}
+
+QEX_HD double fix_double(uint64_t u) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)u);
+#else
+    double d;
+    memcpy(&d, &u, 8);
+    return d;
+#endif
+}
+
+QEX_HD uint32_t fix_mag(double d) { return (uint32_t)(fix_bits(d) >> 32) & 0x7FFFFFFFu; }
+
+// |d| in units of 2^(e - 1023 - 63 + kFixShift), truncated; key = ((e +
+// kFixShift) << 20) | 0xFFFFF with e at least d's exponent field.  Zero (and
+// anything 64 bits below 2^(e - 1023)) gives 0.
+QEX_HD uint64_t fix_abs(uint32_t h, uint32_t l, uint32_t key) {
+    const uint32_t n = (key - (h & 0x7FFFFFFFu)) >> 20;
+#ifdef __CUDA_ARCH__
+    const uint32_t t = __funnelshift_l(l, h, 11);
+#else
+    const uint32_t t = (h << 11) | (l >> 21);
+#endif
+    return fix_shr(((uint64_t)(t | 0x80000000u) << 32) | (l << 11), n);
+}
+
+QEX_HD Digits fix_digits(uint32_t hi, uint32_t lo) {
+    Digits d;
+    d.lo = (int)lo;
+    d.hi = (int)(hi + (lo >> 31));
+#ifdef __CUDA_ARCH__
+    // Opaque from here on: seen through, the products below become 64-bit
+    // multiplications of what the digits were made from.
+    asm("" : "+r"(d.hi), "+r"(d.lo));
+#endif
+    return d;
+}
+
+// Link real: a negative one is complemented instead of negated (one unit of
+// 2^-60 off), a zero of either sign stays 0.
+QEX_HD Digits fix_link_real(double d, uint32_t key) {
+    const uint64_t b = fix_bits(d);
+    const uint32_t h = (uint32_t)(b >> 32);
+    const uint64_t x = fix_abs(h, (uint32_t)b, key);
+    uint32_t hi = (uint32_t)(x >> 32), lo = (uint32_t)x;
+    if (h > 0x80000000u) {
+        hi = ~hi;
+        lo = ~lo;
+    }
+    return fix_digits(hi, lo);
+}
+
+// Vector real times (neg ? -1 : 1), exactly negated.
+QEX_HD uint64_t fix_vec_real(double d, uint32_t key, bool neg) {
+    const uint64_t b = fix_bits(d);
+    const uint32_t h = (uint32_t)(b >> 32);
+    const uint64_t x = fix_abs(h, (uint32_t)b, key);
+    return ((int32_t)h < 0) != neg ? 0 - x : x;
+}
+
+// Sum of the hops so far: value a[.] 2^(e - kFixUnit); re/im of colours 0..2.
+// |a| < 2^62 for up to 8 hops: |U1| |V1| <= 2^56, 6 products a hop.
+constexpr int kFixUnit = 2 * 1023 + 2 * (63 - kFixShift) - 64;
+struct FixSum {
+    int64_t a[6];
+    int e;
+    bool bad;
+};
+
+QEX_HD void fix_clear(FixSum &s) {
+    for (int k = 0; k < 6; ++k) s.a[k] = 0;
+    s.e = 0;
+    s.bad = false;
+}
+
+QEX_HD uint32_t fix_max(uint32_t a, uint32_t b) { return a > b ? a : b; }
+
+// s += (neg ? -1 : 1) U v (DAG: U^+ v).  side(a), a = 0, 1, 2: FP64 work of
+// the caller placed between the integer instructions of the three rows.
+struct NoSide {
+    QEX_HD void operator()(int) const {}
+};
+template <bool DAG, typename Side = NoSide>
+QEX_HD void fix_hop(FixSum &s, const Mat3<double> &u, const Vec3<double> &v, bool neg, const Side &side = Side()) {
+    uint32_t mu = 0, mv = 0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) mu = fix_max(mu, fix_max(fix_mag(u.e[k].re), fix_mag(u.e[k].im)));
+#pragma unroll
+    for (int a = 0; a < 3; ++a) mv = fix_max(mv, fix_max(fix_mag(v.c[a].re), fix_mag(v.c[a].im)));
+    // zeros pass (their digits are 0); other reals out of range do not
+    if (fix_max(mu, mv) >= (uint32_t)kFixHigh << 20) s.bad = true;
+    if (mv < (uint32_t)kFixLow << 20) {
+        uint64_t any = 0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) any |= fix_bits(v.c[a].re) | fix_bits(v.c[a].im);
+        if (any << 1) s.bad = true;  // a sign bit alone is a zero
+        mv = (uint32_t)kFixLow << 20;
+    }
+    if (mu < (uint32_t)kFixLow << 20) {
+        uint64_t any = 0;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) any |= fix_bits(u.e[k].re) | fix_bits(u.e[k].im);
+        if (any << 1) s.bad = true;
+        mu = (uint32_t)kFixLow << 20;
+    }
+    const int eu = (int)(mu >> 20), eh = eu + (int)(mv >> 20);
+    if (eh > s.e) {  // a larger product than the unit allows for: raise the unit
+        const int e = eh + kFixSlack;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) s.a[k] = fix_sar(s.a[k], (uint32_t)(e - s.e));
+        s.e = e;
+    }
+    const uint32_t ku = ((uint32_t)(eu + kFixShift) << 20) | 0xFFFFFu;
+    const uint32_t kv = ((uint32_t)(s.e - eu + kFixShift) << 20) | 0xFFFFFu;
+    Digits vr[3], vi[3], vn[3];  // vn: -vi (DAG: -vr)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const uint64_t re = fix_vec_real(v.c[b].re, kv, neg), im = fix_vec_real(v.c[b].im, kv, neg);
+        vr[b] = fix_digits((uint32_t)(re >> 32), (uint32_t)re);
+        vi[b] = fix_digits((uint32_t)(im >> 32), (uint32_t)im);
+        const uint64_t n = 0 - (DAG ? re : im);
+        vn[b] = fix_digits((uint32_t)(n >> 32), (uint32_t)n);
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        side(a);
+        int64_t hr = s.a[2 * a], hi = s.a[2 * a + 1];
+        int64_t mr = 0x80000000ll, mi = 0x80000000ll;  // the half that rounds the fold below
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int k = DAG ? 3 * b + a : 3 * a + b;
+            const Digits ur = fix_link_real(u.e[k].re, ku), ui = fix_link_real(u.e[k].im, ku);
+            // U: (ur vr - ui vi, ur vi + ui vr);  U^+: (ur vr + ui vi, ur vi - ui vr)
+            const Digits x = DAG ? vi[b] : vn[b], y = DAG ? vn[b] : vr[b];
+            hr = fix_mad(ur.hi, vr[b].hi, hr);
+            mr = fix_mad(ur.hi, vr[b].lo, mr);
+            mr = fix_mad(ur.lo, vr[b].hi, mr);
+            hr = fix_mad(ui.hi, x.hi, hr);
+            mr = fix_mad(ui.hi, x.lo, mr);
+            mr = fix_mad(ui.lo, x.hi, mr);
+            hi = fix_mad(ur.hi, vi[b].hi, hi);
+            mi = fix_mad(ur.hi, vi[b].lo, mi);
+            mi = fix_mad(ur.lo, vi[b].hi, mi);
+            hi = fix_mad(ui.hi, y.hi, hi);
+            mi = fix_mad(ui.hi, y.lo, mi);
+            mi = fix_mad(ui.lo, y.hi, mi);
+        }
+        s.a[2 * a] = fix_mad((int)(mr >> 32), 1, hr);
+        s.a[2 * a + 1] = fix_mad((int)(mi >> 32), 1, hi);
+    }
+}
+
+// The unit of a sum as a double (a power of two in range for a sum that is
+// not bad: exponent fields 2 kFixLow .. 2 kFixHigh + kFixSlack).
+QEX_HD double fix_unit(const FixSum &s) { return fix_double((uint64_t)(uint32_t)(s.e - kFixUnit + 1023) << 52); }
+
+}  // namespace qex
