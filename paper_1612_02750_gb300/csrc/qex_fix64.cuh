@@ -139,37 +139,48 @@ QEX_HD void fix_clear(FixSum &s) {
 
 QEX_HD uint32_t fix_max(uint32_t a, uint32_t b) { return a > b ? a : b; }
 
+// The largest magnitude m (high word) of a link or vector, raised to the
+// smallest accepted one if all of it is zero (any() is the OR of its words);
+// bad is set if it is out of range.
+template <typename Any>
+QEX_HD uint32_t fix_range(uint32_t m, bool &bad, const Any &any) {
+    if (m >= (uint32_t)kFixHigh << 20) bad = true;
+    if (m < (uint32_t)kFixLow << 20) {
+        if (any() << 1) bad = true;  // a sign bit alone is a zero
+        m = (uint32_t)kFixLow << 20;
+    }
+    return m;
+}
+
+QEX_HD uint64_t fix_any(const Vec3<double> &v) {
+    uint64_t any = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) any |= fix_bits(v.c[a].re) | fix_bits(v.c[a].im);
+    return any;
+}
+
 // s += (neg ? -1 : 1) U v (DAG: U^+ v).  side(a), a = 0, 1, 2: FP64 work of
 // the caller placed between the integer instructions of the three rows.
 struct NoSide {
     QEX_HD void operator()(int) const {}
 };
-template <bool DAG, typename Side = NoSide>
+template <bool DAG, int SLACK = kFixSlack, typename Side = NoSide>
 QEX_HD void fix_hop(FixSum &s, const Mat3<double> &u, const Vec3<double> &v, bool neg, const Side &side = Side()) {
     uint32_t mu = 0, mv = 0;
 #pragma unroll
     for (int k = 0; k < 9; ++k) mu = fix_max(mu, fix_max(fix_mag(u.e[k].re), fix_mag(u.e[k].im)));
 #pragma unroll
     for (int a = 0; a < 3; ++a) mv = fix_max(mv, fix_max(fix_mag(v.c[a].re), fix_mag(v.c[a].im)));
-    // zeros pass (their digits are 0); other reals out of range do not
-    if (fix_max(mu, mv) >= (uint32_t)kFixHigh << 20) s.bad = true;
-    if (mv < (uint32_t)kFixLow << 20) {
-        uint64_t any = 0;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) any |= fix_bits(v.c[a].re) | fix_bits(v.c[a].im);
-        if (any << 1) s.bad = true;  // a sign bit alone is a zero
-        mv = (uint32_t)kFixLow << 20;
-    }
-    if (mu < (uint32_t)kFixLow << 20) {
+    mu = fix_range(mu, s.bad, [&] {
         uint64_t any = 0;
 #pragma unroll
         for (int k = 0; k < 9; ++k) any |= fix_bits(u.e[k].re) | fix_bits(u.e[k].im);
-        if (any << 1) s.bad = true;
-        mu = (uint32_t)kFixLow << 20;
-    }
+        return any;
+    });
+    mv = fix_range(mv, s.bad, [&] { return fix_any(v); });
     const int eu = (int)(mu >> 20), eh = eu + (int)(mv >> 20);
     if (eh > s.e) {  // a larger product than the unit allows for: raise the unit
-        const int e = eh + kFixSlack;
+        const int e = eh + SLACK;
 #pragma unroll
         for (int k = 0; k < 6; ++k) s.a[k] = fix_sar(s.a[k], (uint32_t)(e - s.e));
         s.e = e;

@@ -141,3 +141,81 @@ def test_no_less_accurate_than_fmas(q, oracle_mod, naik, links):
         norm = np.sqrt((np.abs(ref) ** 2).sum())
         err = [np.sqrt((np.abs(v - ref) ** 2).sum()) / norm for v in (got, plain)]
         assert err[0] <= 1.05 * err[1], err
+
+
+@pytest.mark.parametrize("naik", [False, True])
+@pytest.mark.parametrize("kind", [0, 1])
+# vectors 2^b: in range, and past it (links, X or Y), where FP64 FMAs take over
+@pytest.mark.parametrize("a,b,c", [(0, 0, 0), (60, -40, 35), (-500, 0, 0), (0, 480, -480), (0, -300, -300)])
+def test_force_scales(q, oracle_mod, naik, kind, a, b, c):
+    """Force and gradient of scaled links and vectors against the oracle's of
+    the unscaled ones (FP64: 1e-13 as in the force's own tests)."""
+    u, w, x = inputs(10, naik)
+    y = inputs(11, naik)[2]
+    lat = q.Lattice(DIMS)
+    fat = q.qex_pack_links(lat, "f64", dev(u * 2.0**a))
+    lng = None if w is None else q.qex_pack_links(lat, "f64", dev(w * 2.0**a))
+    fx = q.qex_pack_field(lat, "f64", 0, dev(x * 2.0**b))
+    fy = q.qex_pack_field(lat, "f64", 1, dev(y * 2.0**c))
+    got = q.qex_force(lat, fat, lng, C3, fx, fy, kind=kind)
+    even = fg.even_mask(DIMS)[..., None]
+    ref = oracle_mod.force(DIMS, u, np.where(even, x, 0), np.where(even, 0, y), w, C3, kind)
+    shift = -b - c - (a if kind == 0 else 0)
+    for g, r in zip(got, ref):
+        if r is not None and g is not None:
+            v = q.qex_unpack_links(lat, "f64", g).cpu().numpy()
+            assert_close(v * 2.0 ** (shift / 2) * 2.0 ** (shift / 2), r, 1e-13, (kind, a, b, c))
+
+
+@pytest.mark.parametrize("value", [np.inf, np.nan, 0.0])
+def test_force_special_values(q, oracle_mod, value):
+    """A colour vector of one site all `value`: the links it reaches are
+    non-finite (or zero), and no others."""
+    u, _, x = inputs(12, False)
+    y = inputs(13, False)[2]
+    x[1, 2, 3, 2] = value  # an even site
+    lat = q.Lattice(DIMS)
+    fat = q.qex_pack_links(lat, "f64", dev(u))
+    g, _ = q.qex_force(lat, fat, None, C3, q.qex_pack_field(lat, "f64", 0, dev(x)),
+                       q.qex_pack_field(lat, "f64", 1, dev(y)), kind=0)
+    got = q.qex_unpack_links(lat, "f64", g).cpu().numpy()
+    even = fg.even_mask(DIMS)
+    xe = np.where(even[..., None], x, 0)
+    with np.errstate(all="ignore"):
+        ref = oracle_mod.force(DIMS, u, xe, np.where(even[..., None], 0, y), None, C3, 0)[0]
+    bad = ~np.isfinite(ref).all((-1, -2))
+    assert np.array_equal(~np.isfinite(got).all((-1, -2)), bad)
+    assert_close(got[~bad], ref[~bad], 1e-13)
+
+
+@pytest.mark.parametrize("links", ["haar", "unit"])
+def test_force_no_less_accurate_than_fp64(q, oracle_mod, links):
+    """F = 2 TA(U G): norm-wise error against extended precision at most that
+    of the oracle's plain FP64 arithmetic."""
+    u, _, x = inputs(14, False)
+    y = inputs(15, False)[2]
+    if links == "unit":
+        u = np.zeros_like(u)
+        u[...] = np.eye(3)
+    even = fg.even_mask(DIMS)
+    x, y = np.where(even[..., None], x, 0), np.where(even[..., None], 0, y)
+    plain = oracle_mod.force(DIMS, u, x, y, None, 0.0, 0)[0]
+    lat = q.Lattice(DIMS)
+    g, _ = q.qex_force(lat, q.qex_pack_links(lat, "f64", dev(u)), None, 0.0, q.qex_pack_field(lat, "f64", 0, dev(x)),
+                       q.qex_pack_field(lat, "f64", 1, dev(y)))
+    got = q.qex_unpack_links(lat, "f64", g).cpu().numpy()
+    z = (x + y).astype(np.clongdouble)  # X on even, Y on odd sites
+    grid = np.indices(fg.lattice_shape(DIMS))
+    xyz = [grid[3], grid[2], grid[1], grid[0]]
+    ref = np.empty(u.shape, np.clongdouble)
+    for mu in range(4):
+        s = (-1.0) ** sum(xyz[:mu], np.zeros(grid[0].shape, int)) * np.where(even, 1.0, -1.0)
+        s = s * np.where((mu == 3) & (xyz[3] + 1 >= DIMS[3]), -1.0, 1.0)
+        there = np.roll(z, -1, axis=3 - mu) * s[..., None]
+        w = (u[..., mu, :, :].astype(np.clongdouble) * there[..., None, :]).sum(-1)
+        m = w[..., :, None] * np.conj(z)[..., None, :]
+        m = m - np.conj(np.swapaxes(m, -1, -2))
+        tr = (m[..., 0, 0] + m[..., 1, 1] + m[..., 2, 2]) / np.longdouble(3)
+        ref[..., mu, :, :] = m - tr[..., None, None] * np.eye(3)
+    err = [np.sqrt((np.abs(v - ref) ** 2).sum() / (np.abs(ref) ** 2).sum()) for v in (got, plain)]
+    assert err[0] <= 1.05 * err[1] and err[1] < 1e-15, err
