@@ -328,9 +328,10 @@ qex_status qex_dot(const qex_lattice *lat, qex_prec prec, const void *a, const v
  * b64, x64: F64 even half fields; x64 holds the initial guess on entry and the
  *   solution on return.  lng64/lng32 NULL = no Naik term.
  * Synchronises the stream before returning (fills stats, may be NULL).
- * Execution: one CUDA graph for the whole solve by default; for a mixed solve
- * with Vh <= 32768 the inner iterations run instead as one persistent
- * cooperative kernel between the reliable updates.  The environment variable
+ * Execution: one CUDA graph for the whole solve by default; on a small lattice
+ * (Vh up to 16384 to 165888, by inner precision and Naik term) the iterations
+ * run instead as one persistent cooperative kernel between the reliable
+ * updates.  The environment variable
  * QEX_CG_MODE = graph | host | fused forces one of the three.
  * Returns QEX_ERR_NOT_CONVERGED after maxiter iterations (x64 holds the last
  * iterate), QEX_ERR_NAN on a NaN/Inf or a non-positive <p, A p>,
@@ -543,7 +544,9 @@ qex_status qex_tune_info(const qex_lattice *lat, qex_prec prec, int naik, int *o
  * other calls does not replace them; qex_tune_info then reports source 4).
  * Use it to reproduce FP64 reduction bits across processes (they are fixed
  * for a given shape) or to run a chosen shape.  A cached CG graph of the
- * lattice is dropped (the device is synchronised first).  Errors:
+ * lattice is dropped (the device is synchronised first).  The
+ * Dslash of a small lattice (four threads a site: Vh up to 28000 to 600000 by
+ * format and Naik term) has one shape and does not follow the pinned one.  Errors:
  * QEX_ERR_ARG (NULL, a value out of range).
  * Paper: no counterpart. */
 qex_status qex_tune_set(const qex_lattice *lat, qex_prec prec, int naik, const int *in);

@@ -10,41 +10,15 @@
 // is folded into the links.
 #include <type_traits>
 #include "qex_dslash64.cuh"
+#include "qex_dslash_params.cuh"
 #include "qex_dslash_site.cuh"
-#include "qex_kernels.cuh"
 
 namespace qex {
-
-template <typename R>
-struct DsParams {
-    Geom g;
-    const R *fat;
-    const R *lng;
-    R c3;
-    int p;              // output parity
-    const R *in;
-    R *out;
-    const R *q;
-    const double *b;
-    R m2;
-    CgScalars *S;
-    int check_halt;
-    const R *r;         // EPI_PUPD
-    R *x;               // EPI_PUPD: iterate that takes the pending alpha p_old (NULL: none)
-    R *pbuf0, *pbuf1;   // p ping-pong
-    int psel;
-    int skip_zero_x;
-    int reverse;        // walk the sites from the last index down
-    int skip_ff;
-    double *partials;
-    unsigned int *counter;
-};
 
 template <typename R, int FMT, bool NAIK, int EPI>
 __global__ void __launch_bounds__(kDslashBlock, DslashMinBlocks<R>::value)
 dslash_kernel(const __grid_constant__ DsParams<R> P) {
     __shared__ double smem[32];
-    __shared__ unsigned int is_last;
     extern __shared__ double2 stage[];  // FP64: the t hops (dslash_site64)
     pdl_trigger();
     pdl_wait();  // everything below may read what earlier kernels wrote
@@ -149,40 +123,7 @@ dslash_kernel(const __grid_constant__ DsParams<R> P) {
             part += d;
         }
     }
-    if constexpr (EPI == EPI_PLAIN || EPI == EPI_PUPD) {
-        return;
-    } else {
-        CgScalars *S = P.S;
-        if (S == nullptr) return;  // uniform over the grid
-
-        // Deterministic grid reduction: block sums -> partials; the last block
-        // to finish sums the partials in index order and updates the CG scalars.
-        const double bs = block_sum(part, smem);
-        if (threadIdx.x == 0) {
-            P.partials[blockIdx.x] = bs;
-            __threadfence();
-            unsigned int t = atomicAdd(P.counter, 1u);
-            is_last = (t == gridDim.x - 1) ? 1u : 0u;
-        }
-        __syncthreads();
-        if (!is_last) return;
-        __threadfence();
-        const double tot = block_sum_partials(P.partials, gridDim.x, smem);
-        if (threadIdx.x != 0) return;
-        *P.counter = 0u;
-        if constexpr (EPI == EPI_NORMAL) {
-            S->pAp = tot;
-            if (!(tot > 0.0) || !isfinite(tot)) {
-                S->error = isfinite(tot) ? 2 : 1;
-                S->halt = 1;
-            } else {
-                S->alpha = S->rr / tot;
-            }
-        } else {
-            // FP64 true residual: accept convergence, or continue with beta from it
-            take_true_residual(S, tot, true);
-        }
-    }
+    if constexpr (EPI == EPI_NORMAL || EPI == EPI_RESID) finish_reduction<R, EPI>(P, part, smem);
 }
 
 // Shape of a Dslash launch: one thread per site, or, for the variants that
@@ -240,6 +181,10 @@ static void launch_t(qex_lattice *lat, const DslashArgs &a, cudaStream_t st) {
     P.skip_ff = a.skip_ff;
     P.partials = lat->partials;
     P.counter = lat->counter;
+    if (lat->vh <= split_limit(std::is_same<R, double>::value, FMT, NAIK)) {
+        launch_split<R>(lat, FMT, NAIK, EPI, P, st);
+        return;
+    }
     int grid, block;
     dslash_shape(lat, a.prec, NAIK, EPI != EPI_PLAIN && EPI != EPI_PUPD && a.S != nullptr, DslashMinBlocks<R>::value,
                  &grid, &block);

@@ -124,7 +124,7 @@ __device__ __forceinline__ Vec3<double> dslash_site64(const Geom &g, const doubl
             t[2].im = (nf3 ? -tf.im : tf.im) + (nb3 ? -tb.im : tb.im);
         }
         bad |= f.bad;
-        const double unit = fix_unit(f);
+        const double unit = fix_unit(f.e);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const double re = fma(unit, (double)f.a[2 * a], t[a].re), im = fma(unit, (double)f.a[2 * a + 1], t[a].im);

@@ -1,0 +1,87 @@
+// qex_dslash_params.cuh -- what the single-field Dslash kernels share: their
+// parameters and the grid reduction that ends the reducing epilogues.
+#pragma once
+
+#include "qex_kernels.cuh"
+
+namespace qex {
+
+template <typename R>
+struct DsParams {
+    Geom g;
+    const R *fat;
+    const R *lng;
+    R c3;
+    int p;              // output parity
+    const R *in;
+    R *out;
+    const R *q;
+    const double *b;
+    R m2;
+    CgScalars *S;
+    int check_halt;
+    const R *r;         // EPI_PUPD
+    R *x;               // EPI_PUPD: iterate that takes the pending alpha p_old (NULL: none)
+    R *pbuf0, *pbuf1;   // p ping-pong
+    int psel;
+    int skip_zero_x;
+    int reverse;        // walk the sites from the last index down
+    int skip_ff;
+    double *partials;
+    unsigned int *counter;
+};
+
+// The grid reduction of EPI_NORMAL and EPI_RESID (part: this thread's sum).
+template <typename R, int EPI>
+__device__ __forceinline__ void finish_reduction(const DsParams<R> &P, double part, double *smem) {
+    __shared__ unsigned int is_last;
+    CgScalars *S = P.S;
+    if (S == nullptr) return;  // uniform over the grid
+
+    // Deterministic grid reduction: block sums -> partials; the last block
+    // to finish sums the partials in index order and updates the CG scalars.
+    const double bs = block_sum(part, smem);
+    if (threadIdx.x == 0) {
+        P.partials[blockIdx.x] = bs;
+        __threadfence();
+        unsigned int t = atomicAdd(P.counter, 1u);
+        is_last = (t == gridDim.x - 1) ? 1u : 0u;
+    }
+    __syncthreads();
+    if (!is_last) return;
+    __threadfence();
+    const double tot = block_sum_partials(P.partials, gridDim.x, smem);
+    if (threadIdx.x != 0) return;
+    *P.counter = 0u;
+    if constexpr (EPI == EPI_NORMAL) {
+        S->pAp = tot;
+        if (!(tot > 0.0) || !isfinite(tot)) {
+            S->error = isfinite(tot) ? 2 : 1;
+            S->halt = 1;
+        } else {
+            S->alpha = S->rr / tot;
+        }
+    } else {
+        // FP64 true residual: accept convergence, or continue with beta from it
+        take_true_residual(S, tot, true);
+    }
+}
+
+// Largest half volume whose Dslash splits each site's directions over four
+// threads (dslash_split.cu); fmt: the fat links' format (qex_dslash_site.cuh).
+// Split / one thread a site, us: FP64 20^4 24.6/28.9, 20 x 22^3 31.5/31.8; with
+// Naik 24^3 x 48 169/174, 32^4 264/258.  FP32 16^2 x 20^2 4.2/4.3, 16^3 x 32
+// 5.0/4.6; with Naik 24^3 x 32 40.8/41.2, 28^4 54.5/51.4.  Two-row FP32 16^4
+// 3.4/3.6, 16^2 x 20^2 4.3/4.1; with Naik 32^4 72.8/76.2, 40^4 183/189 (at HBM
+// both).  16-bit 10 x 14 x 18 x 22 3.3/3.4, 16^4 3.6/3.4; with Naik 16^4
+// 4.9/4.8 (the normal operator 9.7/10.3), 16^3 x 32 7.7/7.1.
+inline int64_t split_limit(bool fp64, int fmt, bool naik) {
+    if (fp64) return naik ? 340000 : 107000;
+    if (fmt >= 2) return naik ? 33000 : 28000;
+    if (fmt == 1) return naik ? 600000 : 42000;
+    return naik ? 230000 : 52000;
+}
+template <typename R>
+void launch_split(const qex_lattice *lat, int fmt, bool naik, int epi, const DsParams<R> &P, cudaStream_t st);
+
+}  // namespace qex

@@ -227,6 +227,6 @@ QEX_HD void fix_hop(FixSum &s, const Mat3<double> &u, const Vec3<double> &v, boo
 
 // The unit of a sum as a double (a power of two in range for a sum that is
 // not bad: exponent fields 2 kFixLow .. 2 kFixHigh + kFixSlack).
-QEX_HD double fix_unit(const FixSum &s) { return fix_double((uint64_t)(uint32_t)(s.e - kFixUnit + 1023) << 52); }
+QEX_HD double fix_unit(int e) { return fix_double((uint64_t)(uint32_t)(e - kFixUnit + 1023) << 52); }
 
 }  // namespace qex
