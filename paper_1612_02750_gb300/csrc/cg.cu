@@ -19,8 +19,8 @@
 // kernel 3 and the update's last kernel set the two conditions.  The loop ends when the true residual meets
 // tol, on the iteration cap, or on a NaN, and in any case after maxiter + 4
 // trips.  Setting QEX_CG_MODE=host instead enqueues batches of iterations
-// from the host and runs the reliable updates between batches.  A mixed
-// solve of a small lattice (Vh <= 32768, or QEX_CG_MODE=fused) runs its inner
+// from the host and runs the reliable updates between batches.  The
+// solve of a small lattice (fused_max_vh, or QEX_CG_MODE=fused) runs its
 // iterations as one persistent cooperative kernel instead (cg_fused.cu), with
 // the reliable updates launched from the host in between.
 //
@@ -44,9 +44,17 @@ void set_count_launches(bool on);
 
 static size_t align256(size_t n) { return (n + 255) & ~size_t(255); }
 
-// Largest half volume that the mixed solve runs as the fused persistent
-// iteration by default (cg_fused.cu).
-constexpr int64_t kFusedAutoMaxVh = 32768;
+// Largest half volume that a solve runs as the fused persistent iteration by
+// default (cg_fused.cu).  Fused / graph, us an iteration: 16-bit 16^3 x 32
+// 22.8/23.4, 20^4 25.7/25.7; with Naik 16^4 20.6/24.9, 16^3 x 32 29.9/29.4; FP32 and
+// two-row FP32 20^4 27.7/30.9 and 25.5/26.9; with Naik 24^4 81/83 and 72/74;
+// FP64 8^4 13.6/22.5, 16^4 37.5/40.1, 16^3 x 32 66.0/61.7; with Naik 12^4 33.4/35.0,
+// 16^4 62.5/62.0.
+static int64_t fused_max_vh(qex_prec inner, bool naik) {
+    if (inner == QEX_F64) return naik ? 16384 : 32768;
+    if (inner == QEX_F32_R12H || inner == QEX_F32_S16) return naik ? 32768 : 65536;
+    return naik ? 165888 : 82944;
+}
 
 struct CgBuffers {
     double *r64, *tmp64, *p64[2], *ap64;
@@ -373,11 +381,11 @@ extern "C" qex_status qex_cg(const qex_lattice *latc, qex_prec inner, const void
     qex_lattice *lat = const_cast<qex_lattice *>(latc);
     if ((st = ensure_scratch(lat))) return st;
     if (!lat->scalars_host2) QEX_CUDA(cudaMallocHost(&lat->scalars_host2, sizeof(CgScalars)));
-    // small lattices default to the persistent fused iteration (1.15-1.3x
-    // faster per iteration up to 16^4); QEX_CG_MODE=graph|host|fused forces
+    // small lattices default to the persistent fused iteration;
+    // QEX_CG_MODE=graph|host|fused forces
     const char *mode = getenv("QEX_CG_MODE");
-    const bool use_fused = mixed && ((mode && strcmp(mode, "fused") == 0) || (!mode && lat->vh <= kFusedAutoMaxVh));
-    const bool use_graph = !(mode && (strcmp(mode, "host") == 0 || use_fused));
+    const bool use_fused = mode ? strcmp(mode, "fused") == 0 : lat->vh <= fused_max_vh(inner, lng64 != nullptr);
+    const bool use_graph = !use_fused && !(mode && strcmp(mode, "host") == 0);
 
     Solve s;
     s.lat = lat;
@@ -479,8 +487,11 @@ extern "C" qex_status qex_cg(const qex_lattice *latc, qex_prec inner, const void
     } else if (!cur.done && !cur.halt && use_fused) {
         // persistent inner iterations, FP64 reliable updates in between
         while (!cur.done && !cur.error) {
-            if ((st = launch_cg_fused(lat, inner, s.fat32, s.lng32, s.c3, s.m2, s.B.xh32, s.B.r32, s.B.p32, s.B.ap32,
-                                      s.B.tmp32, cst)))
+            const FusedVectors v =
+                mixed ? FusedVectors{s.B.xh32, s.B.r32, {s.B.p32[0], s.B.p32[1]}, s.B.ap32, s.B.tmp32}
+                      : FusedVectors{s.x64, s.B.r64, {s.B.p64[0], s.B.p64[1]}, s.B.ap64, s.B.tmp64};
+            if ((st = launch_cg_fused(lat, inner, mixed ? s.fat32 : s.fat64, mixed ? s.lng32 : s.lng64, s.c3, s.m2, v,
+                                      cst)))
                 return st;
             int timed_out = 0, exited = 0;
             if ((st = fused_barrier_status(lat, cst, &timed_out, &exited))) return st;

@@ -1,5 +1,4 @@
-// cg_fused.cu -- the mixed-precision CG iteration of a small lattice as one
-// persistent kernel.
+// cg_fused.cu -- the CG iteration of a small lattice as one persistent kernel.
 //
 // On a small lattice (a few thousand even sites) each of the three kernels of
 // an iteration does a few microseconds of work and the launch, the drain of
@@ -18,9 +17,14 @@
 // three-kernel form computes (the reductions sum the same per-site terms in
 // another block grouping).
 //
-// Grid barriers: arrival counters (per group of 32 blocks, then across the
-// groups) and a generation word, reset by the host before each launch; the
-// last block to arrive bumps the generation.  A wait
+// A site's four directions run on four warps, as in dslash_split.cu (a block
+// is 32 sites per 128 threads), and its colours on three of them, which keep
+// the three phases' vectors of a site at the same thread.
+//
+// Grid barriers: one 64-bit arrival counter, zeroed by the host before each
+// launch and never reset in between; a block adds one (release) and polls until
+// all have come (acquire).  Two L2 round trips, against about five for counters
+// in two levels with a generation word.  A wait
 // that lasts longer than a limit (clock64 cycles, about a second by default;
 // the environment variable QEX_BARRIER_TIMEOUT_CYCLES sets another, which the
 // tests use to make the limit run out) records a timeout in the error word
@@ -30,7 +34,7 @@
 #include <math.h>
 #include <stdlib.h>
 
-#include "qex_dslash_site.cuh"
+#include "qex_dslash_dir.cuh"
 #include "qex_kernels.cuh"
 
 namespace qex {
@@ -42,69 +46,38 @@ struct FusedArgs {
     R c3, m2;
     R *x, *r, *p0, *p1, *ap, *tmp;
     CgScalars *S;
-    double *partials;            // 2 * gridDim.x
-    unsigned int *bar_count;     // barrier counters: top at [0], group g at [(g + 1) * 32]
-    unsigned int *bar_gen;       // barriers completed in this launch
+    double *partials;            // 2 * gridDim.x: block sums of <p, Ap> and ||r||^2
+    unsigned long long *arrived; // blocks that have come to the barriers of this launch; top bit: a wait ran out
     int *bar_err;                // nonzero: a barrier timed out
     unsigned int *exited;        // blocks that have left the kernel
     long long timeout_cycles;    // longest wait at a barrier
 };
 
-constexpr int kFusedBlock = 256;  // most threads per block (launch bounds)
-#ifndef QEX_FUSED_BLOCK
-#define QEX_FUSED_BLOCK 128  // threads per block of a launch (a sweep: 128 beats 256, 64, 32)
-#endif
-#ifndef QEX_FUSED_SPIN_NS
-#define QEX_FUSED_SPIN_NS 0  // sleep between polls of a barrier (0: poll back to back)
-#endif
+// Most threads per block (FP64: 25 KB of sums a block of 256 with the Naik term).
+template <typename R> struct FusedBlock { static constexpr int value = 512; };
+template <> struct FusedBlock<double> { static constexpr int value = 256; };
 constexpr long long kBarrierTimeoutCycles = 2000000000ll;  // default limit: about one second at 2 GHz
+constexpr unsigned long long kBarrierFailed = 1ull << 63;
 
-// Grid barrier number `gen + 1`; false if some block timed out (then every
-// block leaves at its next barrier).  Two levels: a block arrives at the
-// counter of its group of 32 blocks (each counter on its own 128-byte line);
-// the last of a group arrives at the top counter, and the last of those bumps
-// the generation.  Waiting blocks poll the generation with plain loads, so
-// the arrivals' atomics meet no contention from the pollers.
-constexpr int kBarrierGroup = 32;
-constexpr int kBarrierStride = 32;  // unsigned words between counters (128 bytes)
-
-__device__ __forceinline__ bool fused_barrier(unsigned int *counters, unsigned int *gen_word, int *err,
-                                              unsigned int gen, long long timeout_cycles) {
-    __shared__ int ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const int grp = blockIdx.x / kBarrierGroup, ngroups = (gridDim.x + kBarrierGroup - 1) / kBarrierGroup;
-        const unsigned int gsize = min((unsigned int)kBarrierGroup, gridDim.x - grp * kBarrierGroup);
-        unsigned int *gc = counters + (size_t)(grp + 1) * kBarrierStride;
-        bool last = false;
-        if (atomicAdd(gc, 1u) == gsize - 1) {
-            atomicExch(gc, 0u);
-            if (atomicAdd(counters, 1u) == (unsigned int)ngroups - 1) {
-                atomicExch(counters, 0u);
-                __threadfence();
-                atomicExch(gen_word, gen + 1);
-                last = true;
-            }
+// One thread of a block arrives at the grid barrier and waits for `target`
+// arrivals; false if some block's wait ran out (then every block leaves at its
+// next barrier).  The release and the acquire carry what the block's other
+// threads wrote before, and read after, a barrier of the block.
+__device__ __forceinline__ bool arrive_and_wait(unsigned long long *arrived, int *err, unsigned long long target,
+                                                long long timeout_cycles) {
+    asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(arrived) : "memory");
+    const long long t0 = clock64();
+    for (;;) {
+        unsigned long long v;
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(arrived) : "memory");
+        if (v & kBarrierFailed) return false;
+        if (v >= target) return true;
+        if (clock64() - t0 > timeout_cycles) {
+            atomicExch(err, 1);
+            atomicOr(arrived, kBarrierFailed);
+            return false;
         }
-        if (!last) {
-            const volatile unsigned int *gv = gen_word;
-            const volatile int *ev = err;
-            const long long t0 = clock64();
-            while (*gv != gen + 1) {
-                if (*ev != 0) break;
-                if (clock64() - t0 > timeout_cycles) {
-                    atomicExch(err, 1);
-                    break;
-                }
-                if (QEX_FUSED_SPIN_NS > 0) __nanosleep(QEX_FUSED_SPIN_NS);
-            }
-        }
-        __threadfence();
-        ok = *(const volatile int *)err == 0;
     }
-    __syncthreads();
-    return ok != 0;
 }
 
 // Vectors written by this kernel are read back in later phases of the same
@@ -123,30 +96,36 @@ __device__ __forceinline__ Vec3<float> load_vec_cg(const float *base, size_t vh,
     v.c[2].im = u.y;
     return v;
 }
-
-__device__ __forceinline__ Vec3<float> axpy_vec_cg(const float *r, const float *p, float beta, size_t vh, int j) {
-    const Vec3<float> rv = load_vec_cg(r, vh, j), pv = load_vec_cg(p, vh, j);
-    Vec3<float> v;
+__device__ __forceinline__ Vec3<double> load_vec_cg(const double *base, size_t vh, int i) {
+    Vec3<double> v;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        v.c[a].re = fmaf(beta, pv.c[a].re, rv.c[a].re);
-        v.c[a].im = fmaf(beta, pv.c[a].im, rv.c[a].im);
+        const double2 t = __ldcg(reinterpret_cast<const double2 *>(base) + a * vh + i);
+        v.c[a].re = t.x;
+        v.c[a].im = t.y;
     }
     return v;
 }
 
-// Sum of partials[0..n) in index order, returned to every thread of the block.
-__device__ __forceinline__ double fused_total(const double *partials, int n, double *smem) {
-    __shared__ double total;
-    const double s = block_sum_partials(partials, n, smem);
-    if (threadIdx.x == 0) total = s;
-    __syncthreads();
-    return total;
+__device__ __forceinline__ float2 load_colour_cg(const float *f, size_t vh, int a, int i) {
+    return a < 2 ? __ldcg(reinterpret_cast<const float2 *>(f) + 2 * (size_t)i + a)
+                 : __ldcg(reinterpret_cast<const float2 *>(f + 4 * vh) + i);
+}
+__device__ __forceinline__ double2 load_colour_cg(const double *f, size_t vh, int a, int i) {
+    return __ldcg(reinterpret_cast<const double2 *>(f) + a * vh + i);
 }
 
-#ifndef QEX_FUSED_MIN_BLOCKS
-#define QEX_FUSED_MIN_BLOCKS 2  // launch-bounds residency of 256-thread blocks (register cap)
-#endif
+template <typename R>
+__device__ __forceinline__ Vec3<R> axpy_vec_cg(const R *r, const R *p, R beta, size_t vh, int j) {
+    const Vec3<R> rv = load_vec_cg(r, vh, j), pv = load_vec_cg(p, vh, j);
+    Vec3<R> v;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        v.c[a].re = fma(beta, pv.c[a].re, rv.c[a].re);
+        v.c[a].im = fma(beta, pv.c[a].im, rv.c[a].im);
+    }
+    return v;
+}
 
 // Loop state of the solve, identical in every block, kept in shared memory so
 // that it holds no registers during the Dslash phases.
@@ -154,18 +133,61 @@ struct FusedState {
     double rr, beta, rmax2, alpha, pAp;
     double rr_ru;
     int iters, trips, need_ru, ru_ff, error;
+    int ok;  // the last grid barrier was met
 };
 
-template <typename R, int FMT, bool NAIK>
+// Sum of `part` over the grid, in a fixed order: warps, then the block's warps,
+// then the blocks; `then(total)` runs on thread 0.  It is a grid barrier as
+// well.  The first warp does all that follows the block's sum, so the others
+// wait once.  false: some block's wait ran out.
+template <typename Then>
+__device__ __forceinline__ bool fused_sum(double part, double *partials, unsigned long long *arrived, int *err,
+                                          unsigned long long target, long long timeout_cycles, double *smem,
+                                          FusedState &st, const Then &then) {
+    const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
+    if (lane == 0) smem[threadIdx.x >> 5] = part;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        double v = lane < warps ? smem[lane] : 0.0;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        int ok = 1;
+        if (lane == 0) {
+            partials[blockIdx.x] = v;
+            ok = arrive_and_wait(arrived, err, target, timeout_cycles);
+        }
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (ok) {
+            double t = 0.0;
+            for (int k = lane; k < (int)gridDim.x; k += 32) t += __ldcg(partials + k);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+            if (lane == 0) then(t);
+        }
+        if (lane == 0) st.ok = ok;
+    }
+    __syncthreads();
+    return st.ok != 0;
+}
+
+// ONE: every thread has one site at most, and keeps its colour of r, p, x and
+// A p in registers from phase to phase.
+template <typename R, int FMT, bool NAIK, bool ONE>
 __device__ __forceinline__ void cg_fused_body(const FusedArgs<R> &A) {
     __shared__ double smem[32];
     __shared__ FusedState st;
+    __shared__ DirSums<R, FMT, NAIK, FusedBlock<R>::value / 4> sums;
     CgScalars *S = A.S;
     if (S->halt) return;  // uniform
     const Geom &g = A.g;
     const size_t vh = (size_t)g.vh;
     const int nb = gridDim.x;
-    const int stride = nb * blockDim.x;
+    // warp w: sites of group w / 4 of 32, direction (or colour) w % 4
+    const int mu = (threadIdx.x >> 5) & 3, slot = (threadIdx.x >> 7) * 32 + (threadIdx.x & 31);
+    const int first = blockIdx.x * (blockDim.x >> 2) + slot, stride = nb * (blockDim.x >> 2);
+    const int rounds = ONE ? 1 : (g.vh + stride - 1) / stride;
     if (threadIdx.x == 0) {
         st.rr = S->rr;
         st.beta = S->beta;
@@ -179,105 +201,124 @@ __device__ __forceinline__ void cg_fused_body(const FusedArgs<R> &A) {
         st.error = 0;
     }
     __syncthreads();
-    unsigned int gen = 0;
+    unsigned long long target = 0;
+    const bool keeps = ONE && mu < 3 && first < g.vh;
+    typename Pair<R>::type rv, pv, xv, av;  // this thread's r, p, x, A p
+    rv.x = rv.y = R(0);
+    pv = xv = av = rv;
+    if (keeps) {
+        rv = load_colour_cg(A.r, vh, mu, first);
+        pv = load_colour_cg((st.iters & 1) ? A.p1 : A.p0, vh, mu, first);
+        xv = load_colour_cg(A.x, vh, mu, first);
+    }
     for (;;) {
         const int it = st.iters;
         const R *pold = (it & 1) ? A.p1 : A.p0;
         R *pnew = (it & 1) ? A.p0 : A.p1;
-        {   // 1. tmp = D_oe (r + beta p_old); p_new at the thread's own even index
-            const R b = (R)st.beta;
-            for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.vh; i += stride) {
-                const Site s = site_of(g, 1, i);
-                const Vec3<R> acc = dslash_site<R, FMT, NAIK>(g, A.fat, A.lng, A.c3, 1, i, s,
-                                                              [&](int j) { return axpy_vec_cg(A.r, pold, b, vh, j); });
-                store_vec(A.tmp, vh, i, acc);
-                store_vec(pnew, vh, i, axpy_vec_cg(A.r, pold, b, vh, i));
-            }
-        }
-        if (!fused_barrier(A.bar_count, A.bar_gen, A.bar_err, gen++, A.timeout_cycles)) return;
-        {   // 2. A p_new = m^2 p_new - D_eo tmp; <p_new, A p_new>
-            double part = 0.0;
-            for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.vh; i += stride) {
-                const Site s = site_of(g, 0, i);
-                const Vec3<R> acc = dslash_site<R, FMT, NAIK>(
-                    g, A.fat, A.lng, A.c3, 0, i, s, [&](int j) { return load_vec_cg(A.tmp, vh, j); });
-                const Vec3<R> qv = load_vec_cg(pnew, vh, i);
-                Vec3<R> o;
-                R d = R(0);
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    o.c[a].re = fma(A.m2, qv.c[a].re, -acc.c[a].re);
-                    o.c[a].im = fma(A.m2, qv.c[a].im, -acc.c[a].im);
-                    d = fma(qv.c[a].re, o.c[a].re, d);
-                    d = fma(qv.c[a].im, o.c[a].im, d);
+        {   // 1. tmp = D_oe (r + beta p_old); p_new at the site's own even index
+            const R b = (R)st.beta, *const r = A.r;
+            const auto direction = [=](int j) { return axpy_vec_cg(r, pold, b, vh, j); };
+            for (int n = 0, i = first; n < rounds; ++n, i += stride) {
+                const bool mine = i < g.vh;
+                if (mine) {
+                    if (!ONE && mu < 3) {
+                        rv = load_colour_cg(A.r, vh, mu, i);
+                        pv = load_colour_cg(pold, vh, mu, i);
+                    }
+                    sums.put(g, A.fat, A.lng, A.c3, 1, i, mu, slot, direction);
+                    if (mu < 3) {
+                        pv.x = fma(b, pv.x, rv.x);
+                        pv.y = fma(b, pv.y, rv.y);
+                        store_colour(pnew, vh, mu, i, pv);
+                    }
                 }
-                store_vec(A.ap, vh, i, o);
-                part += (double)d;
+                __syncthreads();
+                if (mine && mu < 3)
+                    store_colour(A.tmp, vh, mu, i, sums.get(g, A.fat, A.lng, A.c3, 1, i, mu, slot, direction));
+                if (n + 1 < rounds) __syncthreads();
             }
-            const double bs = block_sum(part, smem);
-            if (threadIdx.x == 0) A.partials[blockIdx.x] = bs;
         }
-        if (!fused_barrier(A.bar_count, A.bar_gen, A.bar_err, gen++, A.timeout_cycles)) return;
-        {
-            const double pAp = fused_total(A.partials, nb, smem);
-            if (threadIdx.x == 0) {
-                st.pAp = pAp;
-                if (!(pAp > 0.0) || !isfinite(pAp))
-                    st.error = isfinite(pAp) ? 2 : 1;
-                else
-                    st.alpha = st.rr / pAp;
+        __syncthreads();
+        if (threadIdx.x == 0) st.ok = arrive_and_wait(A.arrived, A.bar_err, target += nb, A.timeout_cycles);
+        __syncthreads();
+        if (!st.ok) return;
+        {   // 2. A p_new = m^2 p_new - D_eo tmp; <p_new, A p_new> -> alpha
+            double part = 0.0;
+            const R *const tmp = A.tmp;
+            const auto field = [=](int j) { return load_vec_cg(tmp, vh, j); };
+            for (int n = 0, i = first; n < rounds; ++n, i += stride) {
+                const bool mine = i < g.vh;
+                if (mine) {
+                    if (!ONE && mu < 3) pv = load_colour_cg(pnew, vh, mu, i);
+                    sums.put(g, A.fat, A.lng, A.c3, 0, i, mu, slot, field);
+                }
+                __syncthreads();
+                if (mine && mu < 3) {
+                    const auto d = sums.get(g, A.fat, A.lng, A.c3, 0, i, mu, slot, field);
+                    av.x = fma(A.m2, pv.x, -d.x);
+                    av.y = fma(A.m2, pv.y, -d.y);
+                    if (!ONE) store_colour(A.ap, vh, mu, i, av);
+                    part += (double)fma(pv.y, av.y, pv.x * av.x);
+                }
+                if (n + 1 < rounds) __syncthreads();
             }
-            __syncthreads();
+            if (!fused_sum(part, A.partials, A.arrived, A.bar_err, target += nb, A.timeout_cycles, smem, st,
+                           [&](double pAp) {
+                               st.pAp = pAp;
+                               if (!(pAp > 0.0) || !isfinite(pAp))
+                                   st.error = isfinite(pAp) ? 2 : 1;
+                               else
+                                   st.alpha = st.rr / pAp;
+                           }))
+                return;
             if (st.error) break;
         }
         {   // 3. x += alpha p_new; r -= alpha A p_new; ||r||^2
             const R al = (R)st.alpha;
             double part = 0.0;
-            for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.vh; i += stride) {
-                Vec3<R> xv = load_vec_cg(A.x, vh, i), rv = load_vec_cg(A.r, vh, i);
-                const Vec3<R> pv = load_vec_cg(pnew, vh, i), av = load_vec_cg(A.ap, vh, i);
-                R d = R(0);
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    xv.c[a].re = fma(al, pv.c[a].re, xv.c[a].re);
-                    xv.c[a].im = fma(al, pv.c[a].im, xv.c[a].im);
-                    rv.c[a].re = fma(-al, av.c[a].re, rv.c[a].re);
-                    rv.c[a].im = fma(-al, av.c[a].im, rv.c[a].im);
-                    d = fma(rv.c[a].re, rv.c[a].re, d);
-                    d = fma(rv.c[a].im, rv.c[a].im, d);
-                }
-                store_vec(A.x, vh, i, xv);
-                store_vec(A.r, vh, i, rv);
-                part += (double)d;
-            }
-            const double bs = block_sum(part, smem);
-            if (threadIdx.x == 0) A.partials[nb + blockIdx.x] = bs;
-        }
-        if (!fused_barrier(A.bar_count, A.bar_gen, A.bar_err, gen++, A.timeout_cycles)) return;
-        {
-            const double rr_new = fused_total(A.partials + nb, nb, smem);
-            if (threadIdx.x == 0) {
-                st.iters += 1;
-                st.trips += 1;
-                if (!isfinite(rr_new)) {
-                    st.error = 1;
-                } else {
-                    if (rr_new > st.rmax2) st.rmax2 = rr_new;
-                    const bool long_cycle = S->max_cycle > 0 && st.iters - S->ru_iter0 >= S->max_cycle;
-                    if (rr_new <= S->stop2 || rr_new < S->delta2 * st.rmax2 || st.iters >= S->maxiter || long_cycle) {
-                        st.need_ru = 1;  // rr keeps its value: beta then comes from the true residual
-                        st.ru_ff = (S->ff_ok && rr_new > S->stop2 && st.iters < S->maxiter) ? 1 : 0;
-                        st.rr_ru = rr_new;
-                    } else {
-                        st.beta = rr_new / st.rr;
-                        st.rr = rr_new;
+            if (mu < 3) {
+                for (int n = 0, i = first; n < rounds && i < g.vh; ++n, i += stride) {
+                    if (!ONE) {
+                        xv = load_colour_cg(A.x, vh, mu, i);
+                        rv = load_colour_cg(A.r, vh, mu, i);
+                        pv = load_colour_cg(pnew, vh, mu, i);
+                        av = load_colour_cg(A.ap, vh, mu, i);
                     }
+                    xv.x = fma(al, pv.x, xv.x);
+                    xv.y = fma(al, pv.y, xv.y);
+                    rv.x = fma(-al, av.x, rv.x);
+                    rv.y = fma(-al, av.y, rv.y);
+                    if (!ONE) store_colour(A.x, vh, mu, i, xv);
+                    store_colour(A.r, vh, mu, i, rv);
+                    part += (double)fma(rv.y, rv.y, rv.x * rv.x);
                 }
             }
-            __syncthreads();
+            if (!fused_sum(part, A.partials + nb, A.arrived, A.bar_err, target += nb, A.timeout_cycles, smem, st,
+                           [&](double rr_new) {
+                               st.iters += 1;
+                               st.trips += 1;
+                               if (!isfinite(rr_new)) {
+                                   st.error = 1;
+                                   return;
+                               }
+                               if (rr_new > st.rmax2) st.rmax2 = rr_new;
+                               const bool long_cycle = S->max_cycle > 0 && st.iters - S->ru_iter0 >= S->max_cycle;
+                               if (rr_new <= S->stop2 || rr_new < S->delta2 * st.rmax2 || st.iters >= S->maxiter ||
+                                   long_cycle) {
+                                   // rr keeps its value: beta then comes from the true residual
+                                   st.need_ru = 1;
+                                   st.ru_ff = (S->ff_ok && rr_new > S->stop2 && st.iters < S->maxiter) ? 1 : 0;
+                                   st.rr_ru = rr_new;
+                               } else {
+                                   st.beta = rr_new / st.rr;
+                                   st.rr = rr_new;
+                               }
+                           }))
+                return;
             if (st.error || st.need_ru) break;
         }
     }
+    if (keeps) store_colour(A.x, vh, mu, first, xv);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         S->rr = st.rr;
         S->beta = st.beta;
@@ -296,44 +337,53 @@ __device__ __forceinline__ void cg_fused_body(const FusedArgs<R> &A) {
     }
 }
 
-template <typename R, int FMT, bool NAIK>
-__global__ void __launch_bounds__(kFusedBlock, QEX_FUSED_MIN_BLOCKS) cg_fused_kernel(const FusedArgs<R> A) {
-    cg_fused_body<R, FMT, NAIK>(A);
+template <typename R, int FMT, bool NAIK, bool ONE>
+__global__ void __launch_bounds__(FusedBlock<R>::value, 512 / FusedBlock<R>::value)
+cg_fused_kernel(const __grid_constant__ FusedArgs<R> A) {
+    cg_fused_body<R, FMT, NAIK, ONE>(A);
     __syncthreads();
     if (threadIdx.x == 0) atomicAdd(A.exited, 1u);  // every way out of the body ends here
 }
 
 template <typename R, int FMT, bool NAIK>
 static qex_status launch_fused_t(qex_lattice *lat, const FusedArgs<R> &A0, cudaStream_t st) {
-    auto kernel = cg_fused_kernel<R, FMT, NAIK>;
-    int per_sm = 0;
+    // The smallest block that lets one block an SM cover the lattice: fewer
+    // blocks meet sooner at a barrier, smaller ones sum sooner.  12^4 with Naik,
+    // us an iteration: 15.1 (128 threads), 14.5 (256), 13.3 (384), 14.7 (512);
+    // 8^4: 10.1, 10.7, 11.8, 12.9; 16^4: 20.9, 17.5, 17.6, 16.9.
+#ifdef QEX_FUSED_BLOCK
     const int block = QEX_FUSED_BLOCK;
-    QEX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, 0));
-    if (per_sm < 1) {
-        set_error("the fused CG kernel does not fit on an SM");
-        return QEX_ERR_CUDA;
+#else
+    int block = 128;
+    while (block < FusedBlock<R>::value && blocks_for(lat->vh, block / 4) > sm_count()) block += 128;
+#endif
+    const int want = blocks_for(lat->vh, block / 4);
+    auto kernel = cg_fused_kernel<R, FMT, NAIK, true>;
+    int nb = want;
+    for (int one = 1; one >= 0; --one) {
+        if (!one) kernel = cg_fused_kernel<R, FMT, NAIK, false>;
+        int per_sm = 0;
+        QEX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, 0));
+        if (per_sm < 1) {
+            set_error("the fused CG kernel does not fit on an SM");
+            return QEX_ERR_CUDA;
+        }
+        const int cap = per_sm * sm_count();
+        nb = want < cap ? want : cap;
+        if (want <= cap) break;  // one site a thread at most
     }
-    const int want = blocks_for(lat->vh, block);
-    const int cap = per_sm * sm_count();
-    int nb = want < cap ? want : cap;
-    // barrier words after the 2 nb partial sums in the lattice's partials
-    // buffer: the top and group counters (128 bytes apart), then the
-    // generation; the error word is counter[3] of the lattice scratch; all
-    // fresh for every launch
-    const int ngroups = (nb + kBarrierGroup - 1) / kBarrierGroup;
-    const size_t bar_words = (size_t)(ngroups + 1) * kBarrierStride + kBarrierStride;
-    const size_t need = 2 * (size_t)nb + (bar_words * sizeof(unsigned int) + sizeof(double) - 1) / sizeof(double) + 16;
-    if ((size_t)lat->partials_len < need) {
+    // 2 nb partial sums, then the arrival counter, in the lattice's partials
+    // buffer; the error word is counter[3] of the lattice scratch; all fresh for
+    // every launch
+    if ((size_t)lat->partials_len < 2 * (size_t)nb + 32) {
         set_error("internal: partials buffer too small for the fused CG kernel");
         return QEX_ERR_ARG;
     }
-    unsigned int *bar = reinterpret_cast<unsigned int *>(lat->partials + 2 * (size_t)nb + 16);
-    QEX_CUDA(cudaMemsetAsync(bar, 0, bar_words * sizeof(unsigned int), st));
-    QEX_CUDA(cudaMemsetAsync(lat->counter + 3, 0, 2 * sizeof(unsigned int), st));  // error word, exit count
     FusedArgs<R> A = A0;
     A.partials = lat->partials;
-    A.bar_count = bar;
-    A.bar_gen = bar + (size_t)(ngroups + 1) * kBarrierStride;
+    A.arrived = reinterpret_cast<unsigned long long *>(lat->partials + 2 * (size_t)nb + 16);
+    QEX_CUDA(cudaMemsetAsync(A.arrived, 0, sizeof(*A.arrived), st));
+    QEX_CUDA(cudaMemsetAsync(lat->counter + 3, 0, 2 * sizeof(unsigned int), st));  // error word, exit count
     A.bar_err = reinterpret_cast<int *>(lat->counter + 3);
     A.exited = lat->counter + 4;
     A.timeout_cycles = kBarrierTimeoutCycles;
@@ -348,34 +398,35 @@ static qex_status launch_fused_t(qex_lattice *lat, const FusedArgs<R> &A0, cudaS
     return QEX_OK;
 }
 
-template <int FMT>
-static qex_status launch_fused_n(qex_lattice *lat, const FusedArgs<float> &A, bool naik, cudaStream_t st) {
-    return naik ? launch_fused_t<float, FMT, true>(lat, A, st) : launch_fused_t<float, FMT, false>(lat, A, st);
+template <typename R, int FMT>
+static qex_status launch_fused_n(qex_lattice *lat, const FusedVectors &v, const void *fat, const void *lng, double c3,
+                                 double m2, cudaStream_t st) {
+    FusedArgs<R> A = {};
+    A.g = lat->geom;
+    A.fat = (const R *)fat;
+    A.lng = (const R *)lng;
+    A.c3 = (R)c3;
+    A.m2 = (R)m2;
+    A.x = (R *)v.x;
+    A.r = (R *)v.r;
+    A.p0 = (R *)v.p[0];
+    A.p1 = (R *)v.p[1];
+    A.ap = (R *)v.ap;
+    A.tmp = (R *)v.tmp;
+    A.S = lat->scalars;
+    return lng ? launch_fused_t<R, FMT, true>(lat, A, st) : launch_fused_t<R, FMT, false>(lat, A, st);
 }
 
-// One run of the fused iteration kernel (mixed precision only).
-qex_status launch_cg_fused(qex_lattice *lat, qex_prec inner, const void *fat32, const void *lng32, double c3, double m2,
-                           float *x, float *r, float *const p[2], float *ap, float *tmp, cudaStream_t st) {
-    FusedArgs<float> A = {};
-    A.g = lat->geom;
-    A.fat = (const float *)fat32;
-    A.lng = (const float *)lng32;
-    A.c3 = (float)c3;
-    A.m2 = (float)m2;
-    A.x = x;
-    A.r = r;
-    A.p0 = p[0];
-    A.p1 = p[1];
-    A.ap = ap;
-    A.tmp = tmp;
-    A.S = lat->scalars;
-    const bool naik = lng32 != nullptr;
+// One run of the fused iteration kernel.
+qex_status launch_cg_fused(qex_lattice *lat, qex_prec inner, const void *fat, const void *lng, double c3, double m2,
+                           const FusedVectors &v, cudaStream_t st) {
     switch (inner) {
-        case QEX_F32: return launch_fused_n<0>(lat, A, naik, st);
-        case QEX_F32_R12: return launch_fused_n<1>(lat, A, naik, st);
-        case QEX_F32_R12H: return launch_fused_n<2>(lat, A, naik, st);
-        case QEX_F32_S16: return launch_fused_n<3>(lat, A, naik, st);
-        default: set_error("the fused CG iteration is for mixed precision only"); return QEX_ERR_ARG;
+        case QEX_F64: return launch_fused_n<double, 0>(lat, v, fat, lng, c3, m2, st);
+        case QEX_F32: return launch_fused_n<float, 0>(lat, v, fat, lng, c3, m2, st);
+        case QEX_F32_R12: return launch_fused_n<float, 1>(lat, v, fat, lng, c3, m2, st);
+        case QEX_F32_R12H: return launch_fused_n<float, 2>(lat, v, fat, lng, c3, m2, st);
+        case QEX_F32_S16: return launch_fused_n<float, 3>(lat, v, fat, lng, c3, m2, st);
+        default: set_error("unknown inner precision"); return QEX_ERR_ARG;
     }
 }
 
