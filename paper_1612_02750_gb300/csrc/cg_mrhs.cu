@@ -8,9 +8,16 @@
 // on.  A reliable update, requested by any active right-hand side, is done
 // for all active ones: x += x_hat, r = b - A x in FP64, r_hat = (float) r,
 // beta_r = ||r||^2 / rr_r with the previous iterated norm.  An iteration is
-// three kernels (fused direction update + D_oe, normal operator with the
-// per-RHS <p, Ap>, x/r update with the per-RHS norms); the host enqueues them
-// in batches and reads the scalars once per batch.
+// four kernels: direction update (mixed precision: with the iterate's update by
+// the previous step, so that p is read once for both), D_oe, normal operator
+// with the per-RHS <p, Ap>, residual update with the per-RHS norms.  The host
+// enqueues them in batches, one batch ahead of the scalars it reads.
+//
+// What bounds it (24^4, 16 sources, 16-bit links): the Dslash kernels by the
+// L2's bandwidth (about 9 TB/s of neighbour vectors and links), the vector
+// kernels by HBM (every field is 64 MB).  Forming p = r + beta p at each of the
+// eight neighbour reads instead of in a pass of its own gathered two fields:
+// 115 us a D_oe against @@.
 #include <math.h>
 #include <string.h>
 
@@ -21,14 +28,45 @@ namespace qex {
 qex_status check_dslash_args(const qex_lattice *lat, qex_prec prec, const void *fat, const void *lng,
                              const void *in, const void *out);
 
-// blockIdx.y = right-hand side.  x += alpha p_new; r -= alpha ap; ||r||^2;
-// then, in the last block, the lockstep decision: if any active right-hand
-// side asks for a reliable update (or the cap is reached), nobody advances
-// rr/beta and the reliable update takes over; otherwise each advances.
+// blockIdx.y = right-hand side: p = r + beta p and, with x, x += alpha p with
+// the p and alpha of the iteration before (0 after a reliable update).
 template <typename R>
 __global__ void __launch_bounds__(kBlock)
-update_xr_mrhs_kernel(int vh, int nrhs, R *__restrict__ x, R *__restrict__ r, R *pbuf0, R *pbuf1,
-                      const R *__restrict__ ap, MrhsScalars *S, double *partials, unsigned int *counter) {
+update_p_mrhs_kernel(int vh, R *__restrict__ x, const R *__restrict__ r, R *__restrict__ p, const MrhsScalars *S) {
+    if (S->halt) return;  // uniform
+    const int rh = blockIdx.y;
+    if (!S->active[rh]) return;
+    const size_t off = (size_t)rh * 6 * vh;
+    const R beta = (R)S->beta[rh], alpha = x ? (R)S->alpha[rh] : R(0);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < vh; i += gridDim.x * blockDim.x) {
+        const Vec3<R> rv = load_vec(r + off, vh, i);
+        Vec3<R> pv = load_own(p + off, vh, i);
+        if (x) {
+            Vec3<R> xv = load_own(x + off, vh, i);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                xv.c[a].re = fma(alpha, pv.c[a].re, xv.c[a].re);
+                xv.c[a].im = fma(alpha, pv.c[a].im, xv.c[a].im);
+            }
+            store_vec(x + off, vh, i, xv);
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            pv.c[a].re = fma(beta, pv.c[a].re, rv.c[a].re);
+            pv.c[a].im = fma(beta, pv.c[a].im, rv.c[a].im);
+        }
+        store_vec(p + off, vh, i, pv);
+    }
+}
+
+// blockIdx.y = right-hand side.  r -= alpha ap; ||r||^2 (with x, also x +=
+// alpha p); then, in the last block, the lockstep decision: if any active
+// right-hand side asks for a reliable update (or the cap is reached), nobody
+// advances rr/beta and the reliable update takes over; otherwise each advances.
+template <typename R>
+__global__ void __launch_bounds__(kBlock)
+update_r_mrhs_kernel(int vh, int nrhs, R *__restrict__ x, R *__restrict__ r, const R *__restrict__ p,
+                     const R *__restrict__ ap, MrhsScalars *S, double *partials, unsigned int *counter) {
     __shared__ double smem[32];
     __shared__ unsigned int is_last;
     __shared__ double rr_new[kMaxRhs];
@@ -39,19 +77,26 @@ update_xr_mrhs_kernel(int vh, int nrhs, R *__restrict__ x, R *__restrict__ r, R 
     double part = 0.0;
     if (S->active[rh]) {
         const R alpha = (R)S->alpha[rh];
-        const R *p = ((S->iter & 1) ? pbuf0 : pbuf1) + off;
-        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < vh; i += gridDim.x * blockDim.x) {
-            Vec3<R> xv = load_vec(x + off, vh, i), rv = load_vec(r + off, vh, i);
-            const Vec3<R> pv = load_vec(p, vh, i), av = load_vec(ap + off, vh, i);
+        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < vh; k += gridDim.x * blockDim.x) {
+            const int i = vh - 1 - k;  // against the normal operator's order
+            Vec3<R> rv = load_own(r + off, vh, i);
+            const Vec3<R> av = load_vec(ap + off, vh, i);
+            if (x) {
+                Vec3<R> xv = load_own(x + off, vh, i);
+                const Vec3<R> pv = load_vec(p + off, vh, i);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    xv.c[a].re = fma(alpha, pv.c[a].re, xv.c[a].re);
+                    xv.c[a].im = fma(alpha, pv.c[a].im, xv.c[a].im);
+                }
+                store_vec(x + off, vh, i, xv);
+            }
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                xv.c[a].re = fma(alpha, pv.c[a].re, xv.c[a].re);
-                xv.c[a].im = fma(alpha, pv.c[a].im, xv.c[a].im);
                 rv.c[a].re = fma(-alpha, av.c[a].re, rv.c[a].re);
                 rv.c[a].im = fma(-alpha, av.c[a].im, rv.c[a].im);
                 part += (double)(rv.c[a].re * rv.c[a].re + rv.c[a].im * rv.c[a].im);
             }
-            store_vec(x + off, vh, i, xv);
             store_vec(r + off, vh, i, rv);
         }
     }
@@ -89,39 +134,41 @@ update_xr_mrhs_kernel(int vh, int nrhs, R *__restrict__ x, R *__restrict__ r, R 
         }
     }
     __syncthreads();
+    const int iter = S->iter + 1;
+    const bool ru = any_ru || iter >= S->maxiter || (S->max_cycle > 0 && iter - S->ru_iter0 >= S->max_cycle);
+    const bool failed = S->error != 0;
+    __syncthreads();  // every thread has read the scalars that thread 0 writes
+    // a right-hand side a thread
+    const int q = threadIdx.x;
+    if (!failed && !ru && q < nrhs && S->active[q]) {
+        S->beta[q] = rr_new[q] / S->rr[q];
+        S->rr[q] = rr_new[q];
+    }
     if (threadIdx.x == 0) {
-        S->iter += 1;
+        S->iter = iter;
         *counter = 0u;
-        if (S->error) {
-            S->halt = 1;
-        } else if (any_ru || S->iter >= S->maxiter ||
-                   (S->max_cycle > 0 && S->iter - S->ru_iter0 >= S->max_cycle)) {
-            S->need_ru = 1;
-            S->halt = 1;
-        } else {
-            for (int q = 0; q < nrhs; ++q)
-                if (S->active[q]) {
-                    S->beta[q] = rr_new[q] / S->rr[q];
-                    S->rr[q] = rr_new[q];
-                }
-        }
+        if (failed || ru) S->halt = 1;
+        if (!failed && ru) S->need_ru = 1;
     }
 }
 
-// blockIdx.y = right-hand side: x64 += xh32, xh32 = 0 (active ones).
+// blockIdx.y = right-hand side: x64 += xh32 + alpha p (the step that the next
+// direction update would have taken), xh32 = 0 (active ones).
 __global__ void __launch_bounds__(kBlock)
-accum_x_mrhs_kernel(int vh, double *__restrict__ x, float *__restrict__ xh, const MrhsScalars *S) {
+accum_x_mrhs_kernel(int vh, double *__restrict__ x, float *__restrict__ xh, const float *__restrict__ p,
+                    const MrhsScalars *S) {
     const int rh = blockIdx.y;
     if (!S->active[rh]) return;
     const size_t off = (size_t)rh * 6 * vh;
+    const float alpha = (float)S->alpha[rh];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < vh; i += gridDim.x * blockDim.x) {
-        Vec3<double> xv = load_vec(x + off, vh, i);
-        const Vec3<float> hv = load_vec(xh + off, vh, i);
+        Vec3<double> xv = load_own(x + off, vh, i);
+        const Vec3<float> hv = load_own(xh + off, vh, i), pv = load_vec(p + off, vh, i);
         Vec3<float> z;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            xv.c[a].re += (double)hv.c[a].re;
-            xv.c[a].im += (double)hv.c[a].im;
+            xv.c[a].re += (double)fmaf(alpha, pv.c[a].re, hv.c[a].re);
+            xv.c[a].im += (double)fmaf(alpha, pv.c[a].im, hv.c[a].im);
             z.c[a].re = z.c[a].im = 0.f;
         }
         store_vec(x + off, vh, i, xv);
@@ -131,8 +178,9 @@ accum_x_mrhs_kernel(int vh, double *__restrict__ x, float *__restrict__ xh, cons
 
 // blockIdx.y = right-hand side: r32 = (float) r64 (active ones).
 __global__ void __launch_bounds__(kBlock)
-lower_r_mrhs_kernel(int vh, const double *__restrict__ r64, float *__restrict__ r32, const MrhsScalars *S) {
+lower_r_mrhs_kernel(int vh, const double *__restrict__ r64, float *__restrict__ r32, MrhsScalars *S) {
     const int rh = blockIdx.y;
+    if (blockIdx.x == 0 && threadIdx.x == 0) S->alpha[rh] = 0.0;  // no step of the iterate is pending
     if (!S->active[rh]) return;
     const size_t off = (size_t)rh * 6 * vh;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < vh; i += gridDim.x * blockDim.x) {
@@ -191,6 +239,10 @@ norm2_mrhs_kernel(int vh, int nrhs, const double *__restrict__ b, double *__rest
     if (threadIdx.x == 0) *counter = 0u;
 }
 
+// Blocks per SM of the vector kernels over all right-hand sides (24^4, 16
+// sources: 297 us an iteration at 4, 302 at 8; at 64, a pass each, the block
+// sums' FP64 work took as long as the vectors: 92 us a residual update, now 45).
+constexpr int kMrhsBlasPerSm = 4;
 static size_t align256m(size_t n) { return (n + 255) & ~size_t(255); }
 
 }  // namespace qex
@@ -223,15 +275,15 @@ extern "C" qex_status qex_cg_mrhs(const qex_lattice *latc, qex_prec inner, const
     const int vh = (int)lat->vh;
     // nrhs fields back to back, 6*vh reals apart (16-byte aligned: vh is even)
     const size_t f64 = align256m((size_t)vh * 48 * nrhs), f32 = align256m((size_t)vh * 24 * nrhs);
-    // work: r64, tmp64 (+ p64 x2, ap64 in FP64 mode) | xh, r, p x2, ap, tmp (FP32 mode); scalars
-    const size_t need = (mixed ? 2 * f64 + 6 * f32 : 5 * f64) + align256m(sizeof(MrhsScalars));
+    // work: r64, tmp64 (+ p64, ap64 in FP64 mode) | xh, r, p, ap, tmp (FP32 mode); scalars
+    const size_t need = (mixed ? 2 * f64 + 5 * f32 : 4 * f64) + align256m(sizeof(MrhsScalars));
     if ((st = ensure_work(lat, need))) return st;
     char *w = (char *)lat->work;
     double *r64 = (double *)w;
     w += f64;
     double *tmp64 = (double *)w;
     w += f64;
-    void *xi, *ri, *pb[2], *api, *tmpi;
+    void *xi, *ri, *pi, *api, *tmpi;
     const size_t fi = mixed ? f32 : f64;
     if (mixed) {
         xi = w;
@@ -242,9 +294,7 @@ extern "C" qex_status qex_cg_mrhs(const qex_lattice *latc, qex_prec inner, const
         xi = x64;
         ri = r64;
     }
-    pb[0] = w;
-    w += fi;
-    pb[1] = w;
+    pi = w;
     w += fi;
     api = w;
     w += fi;
@@ -265,7 +315,7 @@ extern "C" qex_status qex_cg_mrhs(const qex_lattice *latc, qex_prec inner, const
     init.maxiter = maxiter;
     for (int q = 0; q < nrhs; ++q) init.active[q] = 1;
     MrhsScalars *host = nullptr;
-    QEX_CUDA(cudaMallocHost(&host, sizeof(MrhsScalars)));
+    QEX_CUDA(cudaMallocHost(&host, 2 * sizeof(MrhsScalars)));  // two readback slots
     *host = init;
     cudaEvent_t t0, t1;
     QEX_CUDA(cudaEventCreate(&t0));
@@ -273,11 +323,12 @@ extern "C" qex_status qex_cg_mrhs(const qex_lattice *latc, qex_prec inner, const
     QEX_CUDA(cudaEventRecord(t0, s));
     QEX_CUDA(cudaMemcpyAsync(S, host, sizeof(MrhsScalars), cudaMemcpyHostToDevice, s));
     const size_t fbytes = (size_t)nrhs * vh * (mixed ? 24 : 48);
-    QEX_CUDA(cudaMemsetAsync(pb[0], 0, fbytes, s));
-    QEX_CUDA(cudaMemsetAsync(pb[1], 0, fbytes, s));
+    QEX_CUDA(cudaMemsetAsync(pi, 0, fbytes, s));
     if (mixed) QEX_CUDA(cudaMemsetAsync(xi, 0, fbytes, s));
-    const int nbb = blas_blocks(lat);
-    dim3 bgrid(nbb, nrhs);
+    // about kMrhsBlasPerSm blocks an SM in all, however many right-hand sides
+    int nbb = (sm_count() * kMrhsBlasPerSm + nrhs - 1) / nrhs;
+    if (nbb > blas_blocks(lat)) nbb = blas_blocks(lat);
+    const dim3 bgrid(nbb, nrhs);
     norm2_mrhs_kernel<<<bgrid, kBlock, 0, s>>>(vh, nrhs, (const double *)b64, (double *)x64, S, lat->partials,
                                                lat->counter);
     QEX_CHECK_LAUNCH("norm2_mrhs_kernel");
@@ -289,7 +340,7 @@ extern "C" qex_status qex_cg_mrhs(const qex_lattice *latc, qex_prec inner, const
     a.S = S;
     auto reliable_update = [&]() -> qex_status {
         if (mixed) {
-            accum_x_mrhs_kernel<<<bgrid, kBlock, 0, s>>>(vh, (double *)x64, (float *)xi, S);
+            accum_x_mrhs_kernel<<<bgrid, kBlock, 0, s>>>(vh, (double *)x64, (float *)xi, (const float *)pi, S);
             QEX_CHECK_LAUNCH("accum_x_mrhs_kernel");
         }
         MrhsArgs d = a;
@@ -319,56 +370,80 @@ extern "C" qex_status qex_cg_mrhs(const qex_lattice *latc, qex_prec inner, const
         return QEX_OK;
     };
     auto iteration = [&]() -> qex_status {
+        if (mixed)
+            update_p_mrhs_kernel<float><<<bgrid, kBlock, 0, s>>>(vh, (float *)xi, (const float *)ri, (float *)pi, S);
+        else
+            update_p_mrhs_kernel<double><<<bgrid, kBlock, 0, s>>>(vh, nullptr, (const double *)ri, (double *)pi, S);
+        QEX_CHECK_LAUNCH("update_p_mrhs_kernel");
         MrhsArgs d = a;
         d.prec = inner;
         d.fat = mixed ? fat32 : fat64;
         d.lng = mixed ? lng32 : lng64;
-        d.pbuf[0] = pb[0];
-        d.pbuf[1] = pb[1];
         d.out_parity = 1;
-        d.r = ri;
+        d.in = pi;
         d.out = tmpi;
-        d.epi = EPI_PUPD;
+        d.epi = EPI_PLAIN;
+        // every kernel walks the sites the other way round from the one before,
+        // and meets first what that one left in the L2 (2 %)
+        d.reverse = 1;
         qex_status e;
         if ((e = launch_dslash_mrhs(lat, d, s))) return e;
         d.out_parity = 0;
         d.in = tmpi;
         d.out = api;
         d.epi = EPI_NORMAL;
+        d.q = pi;
+        d.reverse = 0;
         if ((e = launch_dslash_mrhs(lat, d, s))) return e;
         if (mixed)
-            update_xr_mrhs_kernel<float><<<bgrid, kBlock, 0, s>>>(vh, nrhs, (float *)xi, (float *)ri, (float *)pb[0],
-                                                                  (float *)pb[1], (const float *)api, S,
-                                                                  lat->partials, lat->counter);
+            update_r_mrhs_kernel<float><<<bgrid, kBlock, 0, s>>>(vh, nrhs, nullptr, (float *)ri, (const float *)pi,
+                                                                 (const float *)api, S, lat->partials, lat->counter);
         else
-            update_xr_mrhs_kernel<double><<<bgrid, kBlock, 0, s>>>(vh, nrhs, (double *)xi, (double *)ri,
-                                                                   (double *)pb[0], (double *)pb[1],
-                                                                   (const double *)api, S, lat->partials,
-                                                                   lat->counter);
-        QEX_CHECK_LAUNCH("update_xr_mrhs_kernel");
+            update_r_mrhs_kernel<double><<<bgrid, kBlock, 0, s>>>(vh, nrhs, (double *)xi, (double *)ri,
+                                                                  (const double *)pi, (const double *)api, S,
+                                                                  lat->partials, lat->counter);
+        QEX_CHECK_LAUNCH("update_r_mrhs_kernel");
         return QEX_OK;
     };
-    auto fetch = [&]() -> qex_status {
-        QEX_CUDA(cudaMemcpyAsync(host, S, sizeof(MrhsScalars), cudaMemcpyDeviceToHost, s));
-        QEX_CUDA(cudaStreamSynchronize(s));
+    auto fetch = [&](int slot) -> qex_status {
+        QEX_CUDA(cudaMemcpyAsync(host + slot, S, sizeof(MrhsScalars), cudaMemcpyDeviceToHost, s));
+        QEX_CUDA(cudaEventRecord(slot ? lat->ev1 : lat->ev0, s));
+        return QEX_OK;
+    };
+    auto wait = [&](int slot) -> qex_status {
+        QEX_CUDA(cudaEventSynchronize(slot ? lat->ev1 : lat->ev0));
         return QEX_OK;
     };
 
     qex_status result = QEX_OK;
-    if ((st = reliable_update()) || (st = fetch())) {
+    if ((st = reliable_update()) || (st = fetch(0)) || (st = wait(0))) {
         cudaFreeHost(host);
         return st;
     }
     // zero sources: x = 0 exactly
     for (int q = 0; q < nrhs; ++q)
         if (host->bb[q] == 0.0) QEX_CUDA(cudaMemsetAsync((double *)x64 + (size_t)q * 6 * vh, 0, (size_t)vh * 48, s));
-    const int batch = 8;
-    while (!host->error && !host->halt) {
-        for (int k = 0; k < batch; ++k)
-            if ((st = iteration())) break;
-        if (st || (st = fetch())) break;
-        if (host->error || !host->need_ru) continue;
-        if ((st = reliable_update()) || (st = fetch())) break;
+    // Batches of iterations, the next one enqueued before the scalars of the
+    // last are read; the iterations after a halt return at once.
+    const int batch = 4;
+    int slot = 0;  // the slot of the newest scalars that have arrived
+    while (!host[slot].error && !host[slot].halt) {
+        int queued = slot ^ 1;
+        for (int k = 0; k < batch && !st; ++k) st = iteration();
+        if (st || (st = fetch(queued))) break;
+        for (;;) {
+            const int next = queued ^ 1;
+            for (int k = 0; k < batch && !st; ++k) st = iteration();
+            if (st || (st = fetch(next)) || (st = wait(queued))) break;
+            slot = queued;
+            queued = next;
+            if (host[slot].halt) break;
+        }
+        if (st || (st = wait(queued))) break;  // drain the queued batch
+        slot = queued;
+        if (host[slot].error || !host[slot].need_ru) continue;
+        if ((st = reliable_update()) || (st = fetch(0)) || (st = wait(0))) break;
+        slot = 0;
     }
     QEX_CUDA(cudaEventRecord(t1, s));
     QEX_CUDA(cudaEventSynchronize(t1));
@@ -377,9 +452,10 @@ extern "C" qex_status qex_cg_mrhs(const qex_lattice *latc, qex_prec inner, const
     cudaEventDestroy(t0);
     cudaEventDestroy(t1);
     if (!st) {
+        const MrhsScalars &last = host[slot];
         int all = 1;
-        for (int q = 0; q < nrhs; ++q) all &= host->done[q];
-        if (host->error) {
+        for (int q = 0; q < nrhs; ++q) all &= last.done[q];
+        if (last.error) {
             set_error("NaN/Inf or CG breakdown in a multi-RHS solve");
             result = QEX_ERR_NAN;
         } else if (!all) {
@@ -388,11 +464,11 @@ extern "C" qex_status qex_cg_mrhs(const qex_lattice *latc, qex_prec inner, const
         }
         if (stats) {
             for (int q = 0; q < nrhs; ++q) {
-                stats[q].iters = host->iters[q];
-                stats[q].reliable_updates = host->reliable_updates > 0 ? host->reliable_updates - 1 : 0;
-                stats[q].converged = host->done[q];
+                stats[q].iters = last.iters[q];
+                stats[q].reliable_updates = last.reliable_updates > 0 ? last.reliable_updates - 1 : 0;
+                stats[q].converged = last.done[q];
                 stats[q].ff_updates = 0;
-                stats[q].true_rel_resid = host->bb[q] > 0.0 ? sqrt(host->true_rr[q] / host->bb[q]) : 0.0;
+                stats[q].true_rel_resid = last.bb[q] > 0.0 ? sqrt(last.true_rr[q] / last.bb[q]) : 0.0;
                 stats[q].time_ms = ms;
             }
         }

@@ -14,34 +14,26 @@
 namespace qex {
 
 // Thread mapping: one output site per thread and a group of KR right-hand
-// sides per thread (held in registers; KR by precision and epilogue, see
-// MrhsShape): each link is loaded and decoded once per group and applied to
-// all KR vectors.
+// sides per thread (held in registers): each link is loaded and decoded once
+// per group and applied to all KR vectors.
 // A block is 256 sites of one group; linear block b covers site block
 // b / ngroups and group b % ngroups, so the blocks that reuse a link run back
 // to back and find it in L2.
 constexpr int kMrhsBlock = 256;  // threads (sites) per block
 // Right-hand sides per thread (KR) and resident blocks per SM (MINB, the
-// register cap) by precision and epilogue.  The plain Dslash keeps KR = 4 at 2
-// blocks (128 registers: the four accumulators, the four input vectors of a
-// hop and a decoded link; the four independent mat-vecs supply the
-// instruction-level parallelism that the lower occupancy gives up).  The CG
-// epilogues, which also gather the directions or read the q vectors, run
-// faster at KR = 2 and 4 blocks (24^4, 16 sources: the batched mixed CG
-// 0.42 s against 0.46 s).  FP64 takes one at 2 blocks (dslash_site64).
-#ifndef QEX_MRHS_KR_CG
-#define QEX_MRHS_KR_CG 2
-#endif
-#ifndef QEX_MRHS_MIN_BLOCKS_CG
-#define QEX_MRHS_MIN_BLOCKS_CG 4
-#endif
-template <typename R, int EPI>
+// register cap).  FP32: 4 at 2 blocks (128 registers: the four accumulators,
+// the four input vectors of a hop and a decoded link).  What bounds the kernel
+// is the L2's traffic (9 TB/s), and fewer groups read the links less often: the
+// batched mixed CG on 24^4 with 16 sources takes 15 us less an iteration than
+// with the normal operator at KR = 2 and 4 blocks.  FP64 takes one at 2 blocks
+// (dslash_site64).
+template <typename R>
 struct MrhsShape {
-    static constexpr int kr = EPI == EPI_PLAIN ? 4 : QEX_MRHS_KR_CG;
-    static constexpr int minb = EPI == EPI_PLAIN ? 2 : QEX_MRHS_MIN_BLOCKS_CG;
+    static constexpr int kr = 4;
+    static constexpr int minb = 2;
 };
-template <int EPI>
-struct MrhsShape<double, EPI> {
+template <>
+struct MrhsShape<double> {
     static constexpr int kr = 1;
     static constexpr int minb = 2;
 };
@@ -61,15 +53,14 @@ struct MParams {
     R m2;
     MrhsScalars *S;
     int check_halt;
-    const R *r;
-    R *pbuf0, *pbuf1;
+    int reverse;  // walk the site blocks from the last one down
     double *partials;
     unsigned int *counter;
 };
 
 template <typename R, int FMT, bool NAIK, int EPI>
-__global__ void __launch_bounds__(kMrhsBlock, (MrhsShape<R, EPI>::minb)) dslash_mrhs_kernel(const __grid_constant__ MParams<R> P) {
-    constexpr int KR = MrhsShape<R, EPI>::kr;
+__global__ void __launch_bounds__(kMrhsBlock, MrhsShape<R>::minb) dslash_mrhs_kernel(const __grid_constant__ MParams<R> P) {
+    constexpr int KR = MrhsShape<R>::kr;
     __shared__ double wsum[kMrhsBlock / 32][KR];
     __shared__ unsigned int is_last;
     extern __shared__ double2 stage[];  // FP64: the t hops (dslash_site64)
@@ -81,23 +72,16 @@ __global__ void __launch_bounds__(kMrhsBlock, (MrhsShape<R, EPI>::minb)) dslash_
     const int p = P.p;
     const int nsb = (int)((vh + kMrhsBlock - 1) / kMrhsBlock);
     const int total = nsb * P.ngroups;
-    const R *pold = nullptr;
-    R *pnew = nullptr;
-    if (EPI == EPI_PUPD || EPI == EPI_NORMAL) {
-        const int it = S->iter;
-        pold = (it & 1) ? P.pbuf1 : P.pbuf0;
-        pnew = (it & 1) ? P.pbuf0 : P.pbuf1;
-    }
     double part[KR];
 #pragma unroll
     for (int k = 0; k < KR; ++k) part[k] = 0.0;
     // reducing launches have gridDim.x a multiple of ngroups: the group is fixed per block
     for (int bl = blockIdx.x; bl < total; bl += gridDim.x) {
         const int grp = bl % P.ngroups;
-        const int i = (bl / P.ngroups) * kMrhsBlock + threadIdx.x;
+        const int sb = P.reverse ? nsb - 1 - bl / P.ngroups : bl / P.ngroups;
+        const int i = sb * kMrhsBlock + threadIdx.x;
         if (i >= g.vh) continue;
         bool act[KR];
-        R beta[KR];
         size_t off[KR];
         bool any = false;
 #pragma unroll
@@ -106,27 +90,19 @@ __global__ void __launch_bounds__(kMrhsBlock, (MrhsShape<R, EPI>::minb)) dslash_
             act[k] = rh < P.nrhs && (S == nullptr || S->active[rh]);
             any |= act[k];
             off[k] = (size_t)(act[k] ? rh : 0) * fstride;
-            beta[k] = (EPI == EPI_PUPD && act[k]) ? (R)S->beta[rh] : R(0);
         }
         if (!any) continue;
         const Site s = site_of(g, p, i);
         Vec3<R> acc[KR];
         if constexpr (std::is_same<R, double>::value) {
-            double2 *slot = stage + threadIdx.x;
-            if constexpr (EPI == EPI_PUPD)
-                acc[0] = dslash_site64<NAIK>(g, P.fat, P.lng, P.c3, p, i, s,
-                                             Direction64{P.r + off[0], pold + off[0], beta[0], vh}, slot, kMrhsBlock);
-            else
-                acc[0] = dslash_site64<NAIK>(g, P.fat, P.lng, P.c3, p, i, s, Field64{P.in + off[0], vh}, slot,
-                                             kMrhsBlock);
+            acc[0] = dslash_site64<NAIK>(g, P.fat, P.lng, P.c3, p, i, s, Field64{P.in + off[0], vh},
+                                         stage + threadIdx.x, kMrhsBlock);
         } else
         dslash_site_n<R, FMT, NAIK, KR>(g, P.fat, P.lng, P.c3, p, i, s, [&](int j, int k) {
             Vec3<R> v;
             if (!act[k]) {
 #pragma unroll
                 for (int a = 0; a < 3; ++a) v.c[a].re = v.c[a].im = R(0);
-            } else if constexpr (EPI == EPI_PUPD) {
-                v = axpy_vec(P.r + off[k], pold + off[k], beta[k], vh, j);
             } else {
                 v = load_vec(P.in + off[k], vh, j);
             }
@@ -137,11 +113,8 @@ __global__ void __launch_bounds__(kMrhsBlock, (MrhsShape<R, EPI>::minb)) dslash_
             if (!act[k]) continue;
             if constexpr (EPI == EPI_PLAIN) {
                 store_vec(P.out + off[k], vh, i, acc[k]);
-            } else if constexpr (EPI == EPI_PUPD) {
-                store_vec(P.out + off[k], vh, i, acc[k]);
-                store_vec(pnew + off[k], vh, i, axpy_vec(P.r + off[k], pold + off[k], beta[k], vh, i));
             } else if constexpr (EPI == EPI_NORMAL) {
-                const Vec3<R> qv = load_vec(pnew + off[k], vh, i);
+                const Vec3<R> qv = load_vec(P.q + off[k], vh, i);
                 Vec3<R> o;
                 R d = R(0);
 #pragma unroll
@@ -170,7 +143,7 @@ __global__ void __launch_bounds__(kMrhsBlock, (MrhsShape<R, EPI>::minb)) dslash_
             }
         }
     }
-    if constexpr (EPI == EPI_PLAIN || EPI == EPI_PUPD) {
+    if constexpr (EPI == EPI_PLAIN) {
         return;
     } else {
         // per right-hand side of this block's group: a fixed shuffle tree in
@@ -257,7 +230,7 @@ static void launch_m(const qex_lattice *lat, const MrhsArgs &a, cudaStream_t st)
     P.c3 = (R)a.c3;
     P.p = a.out_parity;
     P.nrhs = a.nrhs;
-    constexpr int KR = MrhsShape<R, EPI>::kr;
+    constexpr int KR = MrhsShape<R>::kr;
     P.ngroups = (a.nrhs + KR - 1) / KR;
     P.in = (const R *)a.in;
     P.out = (R *)a.out;
@@ -265,17 +238,15 @@ static void launch_m(const qex_lattice *lat, const MrhsArgs &a, cudaStream_t st)
     P.b = a.b;
     P.m2 = (R)a.m2;
     P.S = a.S;
-    P.check_halt = (a.S && (EPI == EPI_PUPD || EPI == EPI_NORMAL)) ? 1 : 0;
-    P.r = (const R *)a.r;
-    P.pbuf0 = (R *)a.pbuf[0];
-    P.pbuf1 = (R *)a.pbuf[1];
+    P.check_halt = (a.S && EPI != EPI_RESID) ? 1 : 0;
+    P.reverse = a.reverse;
     P.partials = lat->partials;
     P.counter = lat->counter;
     const int nsb = (int)((lat->vh + kMrhsBlock - 1) / kMrhsBlock);
     const int total = nsb * P.ngroups;
     int gx = total;
     if (EPI == EPI_NORMAL || EPI == EPI_RESID) {  // persistent grid, a multiple of ngroups
-        int cap = sm_count() * MrhsShape<R, EPI>::minb;
+        int cap = sm_count() * MrhsShape<R>::minb;
         cap -= cap % P.ngroups;
         if (cap < P.ngroups) cap = P.ngroups;
         gx = total < cap ? total : cap;
@@ -289,8 +260,6 @@ template <typename R, int FMT, bool NAIK>
 static void launch_m_epi(const qex_lattice *lat, const MrhsArgs &a, cudaStream_t st) {
     if (a.epi == EPI_PLAIN)
         launch_m<R, FMT, NAIK, EPI_PLAIN>(lat, a, st);
-    else if (a.epi == EPI_PUPD)
-        launch_m<R, FMT, NAIK, EPI_PUPD>(lat, a, st);
     else if (a.epi == EPI_NORMAL)
         launch_m<R, FMT, NAIK, EPI_NORMAL>(lat, a, st);
     else if constexpr (std::is_same<R, double>::value)

@@ -333,6 +333,30 @@ __device__ __forceinline__ Vec3<float> load_vec(const float *base, size_t vh, in
     return v;
 }
 
+// A vector that the same thread stores back: not through the read-only path.
+__device__ __forceinline__ Vec3<double> load_own(const double *base, size_t vh, int i) {
+    Vec3<double> v;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double2 t = reinterpret_cast<const double2 *>(base)[a * vh + i];
+        v.c[a].re = t.x;
+        v.c[a].im = t.y;
+    }
+    return v;
+}
+__device__ __forceinline__ Vec3<float> load_own(const float *base, size_t vh, int i) {
+    const float4 t = reinterpret_cast<const float4 *>(base)[i];
+    const float2 u = reinterpret_cast<const float2 *>(base + 4 * vh)[i];
+    Vec3<float> v;
+    v.c[0].re = t.x;
+    v.c[0].im = t.y;
+    v.c[1].re = t.z;
+    v.c[1].im = t.w;
+    v.c[2].re = u.x;
+    v.c[2].im = u.y;
+    return v;
+}
+
 __device__ __forceinline__ void store_vec(double *base, size_t vh, int i, const Vec3<double> &v) {
     double2 *b = reinterpret_cast<double2 *>(base) + i;
 #pragma unroll

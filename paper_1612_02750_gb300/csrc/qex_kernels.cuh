@@ -172,12 +172,11 @@ struct MrhsArgs {
     const void *in;       // EPI_PLAIN / EPI_NORMAL / EPI_RESID input fields
     void *out;
     int epi;
-    const void *q;        // EPI_RESID: x fields
+    const void *q;        // EPI_RESID: x fields; EPI_NORMAL: p fields
     const double *b;      // EPI_RESID: b fields (FP64)
     double m2;
     MrhsScalars *S;       // NULL: plain application, no masking
-    const void *r;        // EPI_PUPD
-    void *pbuf[2];        // EPI_PUPD / EPI_NORMAL (q = p_new)
+    int reverse;          // walk the sites from the last one down
 };
 
 qex_status launch_dslash_mrhs(qex_lattice *lat, const MrhsArgs &a, cudaStream_t st);
