@@ -9,28 +9,6 @@
 
 namespace qex {
 
-// Block partial -> partials[]; the last block sums them in index order.
-// Returns true in thread 0 of the last block, with *tot set.
-__device__ __forceinline__ bool grid_sum(double part, double *partials, unsigned int *counter, double *smem,
-                                         double *tot) {
-    __shared__ unsigned int is_last;
-    const double bs = block_sum(part, smem);
-    if (threadIdx.x == 0) {
-        partials[blockIdx.x] = bs;
-        __threadfence();
-        unsigned int t = atomicAdd(counter, 1u);
-        is_last = (t == gridDim.x - 1) ? 1u : 0u;
-    }
-    __syncthreads();
-    if (!is_last) return false;
-    __threadfence();
-    const double s = block_sum_partials(partials, gridDim.x, smem);
-    if (threadIdx.x != 0) return false;
-    *counter = 0u;
-    *tot = s;
-    return true;
-}
-
 template <typename R>
 __device__ __forceinline__ R norm2_site(const Vec3<R> &v) {
     R s = v.c[0].re * v.c[0].re;
@@ -78,6 +56,11 @@ update_xr_kernel(int vh, R *__restrict__ x, R *__restrict__ r, R *pbuf0, R *pbuf
     if (blockIdx.x == 0 && threadIdx.x == 0) set_conditions(ctl, 0u, 0u);
     const R alpha = (R)S->alpha;
     const R *p = (S->iters & 1) ? pbuf0 : pbuf1;  // the new direction
+    // what the last block decides from, read here: its latency is hidden
+    const double rr = S->rr, rmax2_old = S->rmax2, stop2 = S->stop2, delta2 = S->delta2;
+    const int iters = S->iters + 1, trips = S->trips + 1, maxiter = S->maxiter;
+    const bool long_cycle = S->max_cycle > 0 && iters - S->ru_iter0 >= S->max_cycle;
+    const bool ff_ok = S->ff_ok != 0;
     double part = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < vh; i += gridDim.x * blockDim.x) {
         Vec3<R> rv = load_vec(r, vh, i);
@@ -102,30 +85,31 @@ update_xr_kernel(int vh, R *__restrict__ x, R *__restrict__ r, R *pbuf0, R *pbuf
     }
     double rr_new;
     if (!grid_sum(part, partials, counter, smem, &rr_new)) return;
-    S->iters += 1;
-    S->trips += 1;
+    S->iters = iters;
+    S->trips = trips;
     if (!isfinite(rr_new)) {
         S->error = 1;
         S->halt = 1;
         set_conditions(ctl, 0u, 0u);
         return;
     }
-    if (rr_new > S->rmax2) S->rmax2 = rr_new;
-    const bool long_cycle = S->max_cycle > 0 && S->iters - S->ru_iter0 >= S->max_cycle;
-    if (rr_new <= S->stop2 || rr_new < S->delta2 * S->rmax2 || S->iters >= S->maxiter || long_cycle) {
+    const double rmax2 = rr_new > rmax2_old ? rr_new : rmax2_old;
+    S->rmax2 = rmax2;
+    const unsigned int loop = trips < maxiter + 4 ? 1u : 0u;
+    if (rr_new <= stop2 || rr_new < delta2 * rmax2 || iters >= maxiter || long_cycle) {
         // true residual next (reliable update / convergence check); rr keeps
         // the previous value so that beta is formed from the true one; an
         // update that cannot end the solve may run in float-float arithmetic
-        S->ru_ff = (S->ff_ok && rr_new > S->stop2 && S->iters < S->maxiter) ? 1 : 0;
+        S->ru_ff = (ff_ok && rr_new > stop2 && iters < maxiter) ? 1 : 0;
         S->rr_ru = rr_new;
         S->need_ru = 1;
         S->halt = 1;
-        set_conditions(ctl, S->trips < S->maxiter + 4 ? 1u : 0u, 1u);
+        set_conditions(ctl, loop, 1u);
         return;
     }
-    S->beta = rr_new / S->rr;
+    S->beta = rr_new / rr;
     S->rr = rr_new;
-    set_conditions(ctl, S->trips < S->maxiter + 4 ? 1u : 0u, 0u);
+    set_conditions(ctl, loop, 0u);
 }
 
 // p_new = r + beta p_old, buffers by iteration parity

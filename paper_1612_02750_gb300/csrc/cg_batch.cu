@@ -230,10 +230,10 @@ batch_iter_dslash_kernel(const LatDesc *__restrict__ descs, BatchScalars *S, dou
     }
     if constexpr (ROLE == ROLE_K2) {
         if (!last_block_totals(partials, counter, nl, S->astart, tot, nblk)) return;
-        if (threadIdx.x != 0) return;
-        for (int k = 0; k < nl; ++k) {
-            const int l = S->alist[k];
-            const double v = tot[k];
+        // a lattice a thread (one thread for all took about a microsecond each)
+        if ((int)threadIdx.x < nl) {
+            const int l = S->alist[threadIdx.x];
+            const double v = tot[threadIdx.x];
             S->pAp[l] = v;
             if (!(v > 0.0) || !isfinite(v)) {
                 S->error = isfinite(v) ? 2 : 1;
@@ -302,31 +302,40 @@ batch_update_kernel(const LatDesc *__restrict__ descs, BatchScalars *S, double *
         if (threadIdx.x == 0) partials[t] = bs;
     }
     if (!last_block_totals(partials, counter, nl, S->astart, tot, nblk)) return;
-    if (threadIdx.x != 0) return;
-    S->iter += 1;
-    S->trips += 1;
-    int any = 0;
-    for (int k = 0; k < nl; ++k) {
-        const int l = S->alist[k];
-        const double v = tot[k];
-        S->iters[l] += 1;
+    // a lattice a thread
+    const int iter = S->iter + 1;
+    const int trips = S->trips + 1;
+    int need = 0, bad = 0;
+    if ((int)threadIdx.x < nl) {
+        const int l = S->alist[threadIdx.x];
+        const double v = tot[threadIdx.x];
+        const int iters = S->iters[l] + 1;
+        S->iters[l] = iters;
         if (!isfinite(v)) {
-            S->error = 1;
-            continue;
-        }
-        if (v > S->rmax2[l]) S->rmax2[l] = v;
-        if (v <= S->stop2[l] || v < S->delta2 * S->rmax2[l] || S->iter >= S->maxiter ||
-            (S->max_cycle > 0 && S->iters[l] - S->ru_iter0[l] >= S->max_cycle)) {
-            S->need[l] = 1;  // rr keeps its old value: beta comes from the true residual
-            any = 1;
+            bad = 1;
         } else {
-            S->beta[l] = v / S->rr[l];
-            S->rr[l] = v;
+            const double rmax2 = S->rmax2[l] < v ? v : S->rmax2[l];
+            S->rmax2[l] = rmax2;
+            need = v <= S->stop2[l] || v < S->delta2 * rmax2 || iter >= S->maxiter ||
+                   (S->max_cycle > 0 && iters - S->ru_iter0[l] >= S->max_cycle);
+            if (need) {
+                S->need[l] = 1;  // rr keeps its old value: beta comes from the true residual
+            } else {
+                S->beta[l] = v / S->rr[l];
+                S->rr[l] = v;
+            }
         }
     }
+    const int any = __syncthreads_or(need);
+    const int failed = __syncthreads_or(bad) | (S->error != 0);
+    __syncthreads();  // every thread has read what thread 0 writes
+    if (threadIdx.x != 0) return;
+    S->iter = iter;
+    S->trips = trips;
+    if (failed && !S->error) S->error = 1;
     S->any_need = any;
-    S->halt = (any || S->error) ? 1 : 0;
-    const unsigned int go = (!S->error && S->trips < S->maxiter + 4) ? 1u : 0u;
+    S->halt = (any || failed) ? 1 : 0;
+    const unsigned int go = (!failed && trips < S->maxiter + 4) ? 1u : 0u;
     set_conds(ctl, go, (go && any) ? 1u : 0u);
 }
 
@@ -369,28 +378,32 @@ batch_ru_dslash_kernel(const LatDesc *__restrict__ descs, int n, BatchScalars *S
     if constexpr (ROLE == ROLE_RU2) {
         const double bs = block_sum(part, smem);
         if (threadIdx.x == 0) partials[blockIdx.x] = bs;
-        if (threadIdx.x == 0)  // per-lattice tile ranges of the full list
-            for (int k = 0; k <= n; ++k) ident[k] = k < n ? descs[k].tile0 : descs[n - 1].tile0 + descs[n - 1].ntiles;
+        // per-lattice tile ranges of the full list; a lattice a thread
+        const int k = threadIdx.x;
+        if (k <= n) ident[k] = k < n ? descs[k].tile0 : descs[n - 1].tile0 + descs[n - 1].ntiles;
         if (!last_block_totals(partials, counter, n, ident, tot, gridDim.x)) return;
-        if (threadIdx.x != 0) return;
-        for (int k = 0; k < n; ++k) {
-            if (!need[k] || !S->need[k]) continue;
+        int bad = 0;
+        if (k < n && need[k] && S->need[k]) {
             const double v = tot[k];
             S->need[k] = 0;
             S->ru_iter0[k] = S->iters[k];
             S->true_rr[k] = v;
             if (!isfinite(v)) {
-                S->error = 1;
-                continue;
-            }
-            S->beta[k] = S->rr[k] > 0.0 ? v / S->rr[k] : 0.0;
-            S->rr[k] = v;
-            S->rmax2[k] = v;
-            if (v <= S->stop2[k]) {
-                S->done[k] = 1;
-                S->active[k] = 0;
+                bad = 1;
+            } else {
+                const double rr = S->rr[k];
+                S->beta[k] = rr > 0.0 ? v / rr : 0.0;
+                S->rr[k] = v;
+                S->rmax2[k] = v;
+                if (v <= S->stop2[k]) {
+                    S->done[k] = 1;
+                    S->active[k] = 0;
+                }
             }
         }
+        const int failed = __syncthreads_or(bad);  // and the flags above are written
+        if (threadIdx.x != 0) return;
+        if (failed) S->error = 1;
         compact_list(S, descs, n);
         S->nactive = S->nlist;
         S->any_need = 0;

@@ -531,6 +531,47 @@ __device__ __forceinline__ double block_sum_partials(const double *partial, int 
     return block_sum(s, smem);
 }
 
+// Sum of `part` over the grid in a fixed order, in the last block to come
+// here: true in its thread 0, with *tot set.  counter is zero before and after.
+// One release-acquire atomic per block, no separate fences, and two block
+// barriers (three in the last block).  Requires blockDim.x % 32 == 0, <= 1024.
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ bool grid_sum(double part, double *partials, unsigned int *counter, double *smem,
+                                         double *tot) {
+    __shared__ unsigned int is_last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    part = warp_sum(part);
+    if (lane == 0) smem[warp] = part;
+    __syncthreads();
+    if (warp == 0) {
+        const double bs = warp_sum(lane < warps ? smem[lane] : 0.0);
+        if (lane == 0) {
+            partials[blockIdx.x] = bs;
+            unsigned int t;
+            asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;"
+                         : "=r"(t)
+                         : "l"(counter), "r"(gridDim.x - 1)
+                         : "memory");
+            is_last = t == gridDim.x - 1 ? 1u : 0u;
+        }
+    }
+    __syncthreads();
+    if (!is_last) return false;
+    double s = 0.0;
+    for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x) s += __ldcg(partials + k);
+    s = warp_sum(s);
+    if (lane == 0) smem[warp] = s;  // read above before the last barrier
+    __syncthreads();
+    if (warp != 0) return false;
+    s = warp_sum(lane < warps ? smem[lane] : 0.0);
+    *tot = s;
+    return lane == 0;
+}
+
 // ------------------------------------------- programmatic dependent launch
 // A kernel launched with the programmatic-serialization attribute may start
 // while its predecessor in the stream is still finishing: each kernel of the

@@ -34,32 +34,18 @@ struct DsParams {
 // The grid reduction of EPI_NORMAL and EPI_RESID (part: this thread's sum).
 template <typename R, int EPI>
 __device__ __forceinline__ void finish_reduction(const DsParams<R> &P, double part, double *smem) {
-    __shared__ unsigned int is_last;
     CgScalars *S = P.S;
     if (S == nullptr) return;  // uniform over the grid
-
-    // Deterministic grid reduction: block sums -> partials; the last block
-    // to finish sums the partials in index order and updates the CG scalars.
-    const double bs = block_sum(part, smem);
-    if (threadIdx.x == 0) {
-        P.partials[blockIdx.x] = bs;
-        __threadfence();
-        unsigned int t = atomicAdd(P.counter, 1u);
-        is_last = (t == gridDim.x - 1) ? 1u : 0u;
-    }
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    const double tot = block_sum_partials(P.partials, gridDim.x, smem);
-    if (threadIdx.x != 0) return;
-    *P.counter = 0u;
+    const double rr = S->rr;   // before the sum: its latency is hidden there
+    double tot;
+    if (!grid_sum(part, P.partials, P.counter, smem, &tot)) return;
     if constexpr (EPI == EPI_NORMAL) {
         S->pAp = tot;
         if (!(tot > 0.0) || !isfinite(tot)) {
             S->error = isfinite(tot) ? 2 : 1;
             S->halt = 1;
         } else {
-            S->alpha = S->rr / tot;
+            S->alpha = rr / tot;
         }
     } else {
         // FP64 true residual: accept convergence, or continue with beta from it
