@@ -17,7 +17,13 @@
 // L2's bandwidth (about 9 TB/s of neighbour vectors and links), the vector
 // kernels by HBM (every field is 64 MB).  Forming p = r + beta p at each of the
 // eight neighbour reads instead of in a pass of its own gathered two fields:
-// 115 us a D_oe against @@.
+// 115 us a D_oe against 66; an iteration took 355 us, now 267.  Small lattices
+// are bound by the chain of launches and grid reductions, 2 to 3 us each (8^4, 8
+// sources: 32 us an iteration, now 23): each kernel comes up while the one before
+// still runs, the sums take one release-acquire atomic a block, and the last
+// block has read what it decides on before they are in.  A kernel lets the next
+// one up only after its own wait: two kernels waiting at once crowded the running
+// one's blocks onto fewer SMs (12^4, 3 sources: 34.5 us an iteration, now 28.5).
 #include <math.h>
 #include <string.h>
 
@@ -33,11 +39,12 @@ qex_status check_dslash_args(const qex_lattice *lat, qex_prec prec, const void *
 template <typename R>
 __global__ void __launch_bounds__(kBlock)
 update_p_mrhs_kernel(int vh, R *__restrict__ x, const R *__restrict__ r, R *__restrict__ p, const MrhsScalars *S) {
-    if (S->halt) return;  // uniform
+    pdl_wait();
+    pdl_trigger();
     const int rh = blockIdx.y;
-    if (!S->active[rh]) return;
-    const size_t off = (size_t)rh * 6 * vh;
     const R beta = (R)S->beta[rh], alpha = x ? (R)S->alpha[rh] : R(0);
+    if (S->halt | !S->active[rh]) return;  // uniform
+    const size_t off = (size_t)rh * 6 * vh;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < vh; i += gridDim.x * blockDim.x) {
         const Vec3<R> rv = load_vec(r + off, vh, i);
         Vec3<R> pv = load_own(p + off, vh, i);
@@ -68,15 +75,32 @@ __global__ void __launch_bounds__(kBlock)
 update_r_mrhs_kernel(int vh, int nrhs, R *__restrict__ x, R *__restrict__ r, const R *__restrict__ p,
                      const R *__restrict__ ap, MrhsScalars *S, double *partials, unsigned int *counter) {
     __shared__ double smem[32];
-    __shared__ unsigned int is_last;
+    __shared__ bool is_last;
     __shared__ double rr_new[kMaxRhs];
-    __shared__ int any_ru;
+    pdl_wait();
+    pdl_trigger();
+    // what the last block decides on (a right-hand side a thread), read ahead of
+    // the sums: a read after another there costs 0.6 us
+    const int q = threadIdx.x, rh = blockIdx.y;
+    bool mine = false;
+    double rr = 0.0, rmax2 = 0.0, stop2 = 0.0;
+    int iters = 0;
+    if (q < nrhs) {
+        mine = S->active[q] != 0;
+        rr = S->rr[q];
+        rmax2 = S->rmax2[q];
+        stop2 = S->stop2[q];
+        iters = S->iters[q];
+    }
+    const double delta2 = S->delta2;
+    const int iter = S->iter + 1, error = S->error;
+    const bool capped = iter >= S->maxiter || (S->max_cycle > 0 && iter - S->ru_iter0 >= S->max_cycle);
+    const bool on = S->active[rh] != 0;
+    const R alpha = (R)S->alpha[rh];
     if (S->halt) return;  // uniform
-    const int rh = blockIdx.y;
     const size_t off = (size_t)rh * 6 * vh;
     double part = 0.0;
-    if (S->active[rh]) {
-        const R alpha = (R)S->alpha[rh];
+    if (on) {
         for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < vh; k += gridDim.x * blockDim.x) {
             const int i = vh - 1 - k;  // against the normal operator's order
             Vec3<R> rv = load_own(r + off, vh, i);
@@ -100,53 +124,43 @@ update_r_mrhs_kernel(int vh, int nrhs, R *__restrict__ x, R *__restrict__ r, con
             store_vec(r + off, vh, i, rv);
         }
     }
-    const double bs = block_sum(part, smem);
-    if (threadIdx.x == 0) {
-        partials[(size_t)rh * gridDim.x + blockIdx.x] = bs;
-        __threadfence();
-        const unsigned int t = atomicAdd(counter, 1u);
-        is_last = (t == gridDim.x * gridDim.y - 1) ? 1u : 0u;
-    }
+    const int lane = q & 31, warp = q >> 5, nw = blockDim.x >> 5;
+    part = warp_sum(part);
+    if (lane == 0) smem[warp] = part;
     __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    if (threadIdx.x == 0) any_ru = 0;
-    __syncthreads();
-    // one warp per right-hand side, fixed order over the blocks
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int q = warp; q < nrhs; q += nw) {
-        double v = 0.0;
-        for (int bx = lane; bx < (int)gridDim.x; bx += 32) v += __ldcg(partials + (size_t)q * gridDim.x + bx);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (warp == 0) {
+        const double bs = warp_sum(lane < nw ? smem[lane] : 0.0);
         if (lane == 0) {
-            rr_new[q] = v;
-            if (S->active[q]) {
-                S->iters[q] += 1;
-                if (!isfinite(v)) {
-                    S->error = 1;
-                    atomicOr(&any_ru, 1);
-                } else {
-                    if (v > S->rmax2[q]) S->rmax2[q] = v;
-                    if (v <= S->stop2[q] || v < S->delta2 * S->rmax2[q]) atomicOr(&any_ru, 1);
-                }
-            }
+            partials[(size_t)rh * gridDim.x + blockIdx.x] = bs;
+            is_last = arrive_last(counter, gridDim.x * gridDim.y);
         }
     }
     __syncthreads();
-    const int iter = S->iter + 1;
-    const bool ru = any_ru || iter >= S->maxiter || (S->max_cycle > 0 && iter - S->ru_iter0 >= S->max_cycle);
-    const bool failed = S->error != 0;
-    __syncthreads();  // every thread has read the scalars that thread 0 writes
-    // a right-hand side a thread
-    const int q = threadIdx.x;
-    if (!failed && !ru && q < nrhs && S->active[q]) {
-        S->beta[q] = rr_new[q] / S->rr[q];
-        S->rr[q] = rr_new[q];
+    if (!is_last) return;
+    // one warp per right-hand side, fixed order over the blocks
+    for (int k = warp; k < nrhs; k += nw) {
+        double v = 0.0;
+#pragma unroll 4
+        for (int bx = lane; bx < (int)gridDim.x; bx += 32) v += __ldcg(partials + (size_t)k * gridDim.x + bx);
+        v = warp_sum(v);
+        if (lane == 0) rr_new[k] = v;
     }
-    if (threadIdx.x == 0) {
+    __syncthreads();
+    const double v = mine ? rr_new[q] : 0.0;
+    const bool failed = __syncthreads_or(mine && !isfinite(v)) || error;
+    if (v > rmax2) rmax2 = v;
+    const bool ru = __syncthreads_or(mine && (v <= stop2 || v < delta2 * rmax2)) || capped;
+    if (mine) {
+        S->iters[q] = iters + 1;
+        S->rmax2[q] = rmax2;
+        if (!failed && !ru) {
+            S->beta[q] = v / rr;
+            S->rr[q] = v;
+        }
+    }
+    if (q == 0) {
         S->iter = iter;
-        *counter = 0u;
+        if (failed) S->error = error ? error : 1;
         if (failed || ru) S->halt = 1;
         if (!failed && ru) S->need_ru = 1;
     }
@@ -370,12 +384,17 @@ extern "C" qex_status qex_cg_mrhs(const qex_lattice *latc, qex_prec inner, const
         return QEX_OK;
     };
     auto iteration = [&]() -> qex_status {
+        // linked by programmatic launches: the next kernel's blocks come up while
+        // this one's last are still running
         if (mixed)
-            update_p_mrhs_kernel<float><<<bgrid, kBlock, 0, s>>>(vh, (float *)xi, (const float *)ri, (float *)pi, S);
+            launch_k(update_p_mrhs_kernel<float>, bgrid, dim3(kBlock), 0, s, true, vh, (float *)xi, (const float *)ri,
+                     (float *)pi, (const MrhsScalars *)S);
         else
-            update_p_mrhs_kernel<double><<<bgrid, kBlock, 0, s>>>(vh, nullptr, (const double *)ri, (double *)pi, S);
+            launch_k(update_p_mrhs_kernel<double>, bgrid, dim3(kBlock), 0, s, true, vh, (double *)nullptr,
+                     (const double *)ri, (double *)pi, (const MrhsScalars *)S);
         QEX_CHECK_LAUNCH("update_p_mrhs_kernel");
         MrhsArgs d = a;
+        d.pdl = 1;
         d.prec = inner;
         d.fat = mixed ? fat32 : fat64;
         d.lng = mixed ? lng32 : lng64;
@@ -396,12 +415,11 @@ extern "C" qex_status qex_cg_mrhs(const qex_lattice *latc, qex_prec inner, const
         d.reverse = 0;
         if ((e = launch_dslash_mrhs(lat, d, s))) return e;
         if (mixed)
-            update_r_mrhs_kernel<float><<<bgrid, kBlock, 0, s>>>(vh, nrhs, nullptr, (float *)ri, (const float *)pi,
-                                                                 (const float *)api, S, lat->partials, lat->counter);
+            launch_k(update_r_mrhs_kernel<float>, bgrid, dim3(kBlock), 0, s, true, vh, nrhs, (float *)nullptr,
+                     (float *)ri, (const float *)pi, (const float *)api, S, lat->partials, lat->counter);
         else
-            update_r_mrhs_kernel<double><<<bgrid, kBlock, 0, s>>>(vh, nrhs, (double *)xi, (double *)ri,
-                                                                  (const double *)pi, (const double *)api, S,
-                                                                  lat->partials, lat->counter);
+            launch_k(update_r_mrhs_kernel<double>, bgrid, dim3(kBlock), 0, s, true, vh, nrhs, (double *)xi,
+                     (double *)ri, (const double *)pi, (const double *)api, S, lat->partials, lat->counter);
         QEX_CHECK_LAUNCH("update_r_mrhs_kernel");
         return QEX_OK;
     };

@@ -531,6 +531,18 @@ __device__ __forceinline__ double block_sum_partials(const double *partial, int 
     return block_sum(s, smem);
 }
 
+// One arrival at a grid's counter, which the last one leaves at zero again: what
+// this thread (and those that it has synchronised with) wrote is released to the
+// block for which it returns true.
+__device__ __forceinline__ bool arrive_last(unsigned int *counter, unsigned int blocks) {
+    unsigned int t;
+    asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;"
+                 : "=r"(t)
+                 : "l"(counter), "r"(blocks - 1)
+                 : "memory");
+    return t == blocks - 1;
+}
+
 // Sum of `part` over the grid in a fixed order, in the last block to come
 // here: true in its thread 0, with *tot set.  counter is zero before and after.
 // One release-acquire atomic per block, no separate fences, and two block
@@ -542,7 +554,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 __device__ __forceinline__ bool grid_sum(double part, double *partials, unsigned int *counter, double *smem,
                                          double *tot) {
-    __shared__ unsigned int is_last;
+    __shared__ bool is_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     part = warp_sum(part);
     if (lane == 0) smem[warp] = part;
@@ -551,12 +563,7 @@ __device__ __forceinline__ bool grid_sum(double part, double *partials, unsigned
         const double bs = warp_sum(lane < warps ? smem[lane] : 0.0);
         if (lane == 0) {
             partials[blockIdx.x] = bs;
-            unsigned int t;
-            asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;"
-                         : "=r"(t)
-                         : "l"(counter), "r"(gridDim.x - 1)
-                         : "memory");
-            is_last = t == gridDim.x - 1 ? 1u : 0u;
+            is_last = arrive_last(counter, gridDim.x);
         }
     }
     __syncthreads();

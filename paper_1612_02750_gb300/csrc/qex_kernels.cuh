@@ -177,6 +177,7 @@ struct MrhsArgs {
     double m2;
     MrhsScalars *S;       // NULL: plain application, no masking
     int reverse;          // walk the sites from the last one down
+    int pdl;              // programmatic dependent launch
 };
 
 qex_status launch_dslash_mrhs(qex_lattice *lat, const MrhsArgs &a, cudaStream_t st);
