@@ -131,27 +131,45 @@ __device__ __forceinline__ void set_conds(const GraphCtl &ctl, unsigned int loop
 // (one warp per lattice) into tot[].
 __device__ __forceinline__ bool last_block_totals(double *partials, unsigned int *counter, int nl, const int *start,
                                                   double *tot, unsigned int nblocks) {
-    __shared__ unsigned int is_last;
+    __shared__ bool is_last;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned int t = atomicAdd(counter, 1u);
-        is_last = (t == nblocks - 1) ? 1u : 0u;
-    }
+    if (threadIdx.x == 0) is_last = arrive_last(counter, nblocks);
     __syncthreads();
     if (!is_last) return false;
-    __threadfence();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     for (int k = warp; k < nl; k += nw) {
         double v = 0.0;
+#pragma unroll 4
         for (int j = start[k] + lane; j < start[k + 1]; j += 32) v += __ldcg(partials + j);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        v = warp_sum(v);
         if (lane == 0) tot[k] = v;
     }
     __syncthreads();
-    if (threadIdx.x == 0) *counter = 0u;
     return true;
+}
+
+// What a kernel of the iteration needs of the scalars to find its work, read at
+// once: one after another, each costs an L2 latency of 0.6 us.  The caller
+// synchronises the block before it reads the arrays.  With the sums' single
+// atomic a block, and the last block's reads ahead of them, 8^4 and 12^4 together
+// take 61 ms, 73 before; 8^4 to 32^4, eight lattices, 272 ms, 295 before.
+// (Programmatic launches give the small ones 2 ms more, but put the next kernel's
+// waiting blocks in the large ones' way: 300 ms.)
+struct WorkList {
+    int bstart[kMaxRhs + 1], astart[kMaxRhs + 1], alist[kMaxRhs];
+};
+struct WorkScalars {
+    int halt, nl, spt, it;
+};
+__device__ __forceinline__ WorkScalars read_work(const BatchScalars *S, WorkList &w) {
+    static_assert(kTile > kMaxRhs, "an entry a thread");
+    const int t = threadIdx.x;
+    if (t <= kMaxRhs) {
+        w.bstart[t] = S->bstart[t];
+        w.astart[t] = S->astart[t];
+    }
+    if (t < kMaxRhs) w.alist[t] = S->alist[t];
+    return {S->halt, S->nlist, S->spt, S->iter};
 }
 
 // Iteration Dslash kernels: persistent grid over the compacted tile list.
@@ -160,24 +178,25 @@ __global__ void __launch_bounds__(kTile, BatchMinBlocks<R>::value)
 batch_iter_dslash_kernel(const LatDesc *__restrict__ descs, BatchScalars *S, double *partials, unsigned int *counter) {
     __shared__ double smem[32];
     __shared__ double tot[kMaxRhs];
+    __shared__ WorkList L;
     extern __shared__ double2 stage[];  // FP64: the t hops (dslash_site64)
-    if (S->halt) return;  // uniform over the grid
-    const int nl = S->nlist;
-    const int nitems = S->bstart[nl];
-    const int spt = S->spt;
-    const int it = S->iter;
+    const WorkScalars ws = read_work(S, L);
+    __syncthreads();
+    if (ws.halt) return;  // uniform over the grid
+    const int nl = ws.nl, spt = ws.spt, it = ws.it;
+    const int nitems = L.bstart[nl];
     // blocks beyond the running work items leave at once (the last running
     // lattice can be a few items against a grid sized for all of them)
     const unsigned int nblk = nitems < (int)gridDim.x ? (unsigned int)nitems : gridDim.x;
     if (blockIdx.x >= nblk) return;
     for (int w = blockIdx.x; w < nitems; w += gridDim.x)
     for (int q = 0; q < spt; ++q) {
-        const int k = find_start(S->bstart, nl, w);
-        const int l = S->alist[k];
+        const int k = find_start(L.bstart, nl, w);
+        const int l = L.alist[k];
         const LatDesc &D = descs[l];
-        const int grp = (w - S->bstart[k]) * spt + q;  // group within the lattice
+        const int grp = (w - L.bstart[k]) * spt + q;  // group within the lattice
         if (grp >= D.ntiles) break;                     // uniform over the block
-        const int t = S->astart[k] + grp;               // group in the compacted list
+        const int t = L.astart[k] + grp;               // group in the compacted list
         const Geom &g = D.g;
         const size_t vh = (size_t)g.vh;
         const int i = grp * kTile + threadIdx.x;
@@ -229,17 +248,19 @@ batch_iter_dslash_kernel(const LatDesc *__restrict__ descs, BatchScalars *S, dou
         }
     }
     if constexpr (ROLE == ROLE_K2) {
-        if (!last_block_totals(partials, counter, nl, S->astart, tot, nblk)) return;
         // a lattice a thread (one thread for all took about a microsecond each)
-        if ((int)threadIdx.x < nl) {
-            const int l = S->alist[threadIdx.x];
+        const bool mine = (int)threadIdx.x < nl;
+        const int l = mine ? L.alist[threadIdx.x] : 0;
+        const double rr = mine ? S->rr[l] : 0.0;  // read ahead of the sums
+        if (!last_block_totals(partials, counter, nl, L.astart, tot, nblk)) return;
+        if (mine) {
             const double v = tot[threadIdx.x];
             S->pAp[l] = v;
             if (!(v > 0.0) || !isfinite(v)) {
                 S->error = isfinite(v) ? 2 : 1;
                 S->halt = 1;
             } else {
-                S->alpha[l] = S->rr[l] / v;
+                S->alpha[l] = rr / v;
             }
         }
     }
@@ -253,7 +274,10 @@ batch_update_kernel(const LatDesc *__restrict__ descs, BatchScalars *S, double *
                     const GraphCtl ctl) {
     __shared__ double smem[32];
     __shared__ double tot[kMaxRhs];
-    if (S->halt) {
+    __shared__ WorkList L;
+    const WorkScalars ws = read_work(S, L);
+    __syncthreads();
+    if (ws.halt) {
         // an earlier iteration of the same graph trip asked for a reliable
         // update (keep its conditions) or the batch stopped (end the loop)
         if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -265,25 +289,24 @@ batch_update_kernel(const LatDesc *__restrict__ descs, BatchScalars *S, double *
     }
     // fail-safe: stop unless the last block sets the conditions again
     if (blockIdx.x == 0 && threadIdx.x == 0) set_conds(ctl, 0u, 0u);
-    const int nl = S->nlist;
-    const int nitems = S->bstart[nl];
-    const int spt = S->spt;
+    const int nl = ws.nl, spt = ws.spt;
+    const int nitems = L.bstart[nl];
     const unsigned int nblk = nitems < (int)gridDim.x ? (unsigned int)nitems : gridDim.x;
     if (blockIdx.x >= nblk) return;  // a running list is never empty here (an empty one halts)
     for (int w = blockIdx.x; w < nitems; w += gridDim.x)
     for (int q = 0; q < spt; ++q) {
-        const int k = find_start(S->bstart, nl, w);
-        const int l = S->alist[k];
+        const int k = find_start(L.bstart, nl, w);
+        const int l = L.alist[k];
         const LatDesc &D = descs[l];
-        const int grp = (w - S->bstart[k]) * spt + q;
+        const int grp = (w - L.bstart[k]) * spt + q;
         if (grp >= D.ntiles) break;  // uniform over the block
-        const int t = S->astart[k] + grp;
+        const int t = L.astart[k] + grp;
         const size_t vh = (size_t)D.g.vh;
         const int i = grp * kTile + threadIdx.x;
         double part = 0.0;
         if (i < D.g.vh) {
             const R alpha = (R)S->alpha[l];
-            const R *p = (const R *)((S->iter & 1) ? D.p0 : D.p1);
+            const R *p = (const R *)((ws.it & 1) ? D.p0 : D.p1);
             R *x = (R *)D.xi, *r = (R *)D.ri;
             Vec3<R> xv = load_vec(x, vh, i), rv = load_vec(r, vh, i);
             const Vec3<R> pv = load_vec(p, vh, i), av = load_vec((const R *)D.api, vh, i);
@@ -301,41 +324,40 @@ batch_update_kernel(const LatDesc *__restrict__ descs, BatchScalars *S, double *
         const double bs = block_sum(part, smem);
         if (threadIdx.x == 0) partials[t] = bs;
     }
-    if (!last_block_totals(partials, counter, nl, S->astart, tot, nblk)) return;
-    // a lattice a thread
-    const int iter = S->iter + 1;
-    const int trips = S->trips + 1;
+    // a lattice a thread; what it decides on is read ahead of the sums
+    const bool mine = (int)threadIdx.x < nl;
+    const int l = mine ? L.alist[threadIdx.x] : 0;
+    const int iter = ws.it + 1, trips = S->trips + 1, error = S->error, maxiter = S->maxiter, cap = S->max_cycle;
+    const int iters = S->iters[l] + 1, ru_iter0 = S->ru_iter0[l];
+    const double rr = S->rr[l], old_max = S->rmax2[l], stop2 = S->stop2[l], delta2 = S->delta2;
+    if (!last_block_totals(partials, counter, nl, L.astart, tot, nblk)) return;
     int need = 0, bad = 0;
-    if ((int)threadIdx.x < nl) {
-        const int l = S->alist[threadIdx.x];
+    if (mine) {
         const double v = tot[threadIdx.x];
-        const int iters = S->iters[l] + 1;
         S->iters[l] = iters;
         if (!isfinite(v)) {
             bad = 1;
         } else {
-            const double rmax2 = S->rmax2[l] < v ? v : S->rmax2[l];
+            const double rmax2 = old_max < v ? v : old_max;
             S->rmax2[l] = rmax2;
-            need = v <= S->stop2[l] || v < S->delta2 * rmax2 || iter >= S->maxiter ||
-                   (S->max_cycle > 0 && iters - S->ru_iter0[l] >= S->max_cycle);
+            need = v <= stop2 || v < delta2 * rmax2 || iter >= maxiter || (cap > 0 && iters - ru_iter0 >= cap);
             if (need) {
                 S->need[l] = 1;  // rr keeps its old value: beta comes from the true residual
             } else {
-                S->beta[l] = v / S->rr[l];
+                S->beta[l] = v / rr;
                 S->rr[l] = v;
             }
         }
     }
     const int any = __syncthreads_or(need);
-    const int failed = __syncthreads_or(bad) | (S->error != 0);
-    __syncthreads();  // every thread has read what thread 0 writes
+    const int failed = __syncthreads_or(bad) | (error != 0);
     if (threadIdx.x != 0) return;
     S->iter = iter;
     S->trips = trips;
-    if (failed && !S->error) S->error = 1;
+    if (failed && !error) S->error = 1;
     S->any_need = any;
     S->halt = (any || failed) ? 1 : 0;
-    const unsigned int go = (!failed && trips < S->maxiter + 4) ? 1u : 0u;
+    const unsigned int go = (!failed && trips < maxiter + 4) ? 1u : 0u;
     set_conds(ctl, go, (go && any) ? 1u : 0u);
 }
 
