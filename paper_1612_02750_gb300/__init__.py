@@ -145,6 +145,9 @@ def _prec(p) -> int:
         raise ValueError(f"unknown precision {p!r}") from None
 
 
+# What one call of a small operator costs the host (8^4, FP64 normal operator) is
+# as long as its kernels: pointers and streams go to the library as plain ints, and
+# the stream's handle is asked for without building a Stream object around it.
 def _ptr(t):
     if t is None:
         return None
@@ -154,13 +157,13 @@ def _ptr(t):
         raise ValueError("tensor must live on a CUDA device")
     if not t.is_contiguous():
         raise ValueError("tensor must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream=None):
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 class Lattice:
