@@ -555,8 +555,9 @@ qex_status qex_tune_set(const qex_lattice *lat, qex_prec prec, int naik, const i
  * per FMA): *fp64_gflops (double) and *fp32_gflops (float, scalar FMA), from
  * fixed-trip FMA chains over several resident waves, timed with CUDA events
  * on `stream` (best of five bursts of a few ms; allocates and frees 512 KB of scratch;
- * synchronises the stream).  The FP64 rate bounds the FP64 Dslash on a GPU
- * whose FP64 units are few (GB300: about 1.2 TFLOP/s, 288 FP64 FMAs per site).
+ * synchronises the stream).  The FP64 rate (GB300: about 1.2 TFLOP/s) is
+ * what the FP64 Dslash avoids: a site's hops stand for 288 FP64 FMAs, and three
+ * quarters of them run in fixed point on the integer pipe.
  * Errors: QEX_ERR_ARG (NULL), QEX_ERR_CUDA.
  * Paper: no counterpart (a measurement of the hardware). */
 qex_status qex_fma_rates(double *fp64_gflops, double *fp32_gflops, void *stream);

@@ -1,6 +1,6 @@
 // probe.cu -- qex_fma_rates: the FP64 and FP32 fused multiply-add rates of
-// the current GPU, the ceilings behind the FP64 Dslash (FP64-ALU bound on a
-// GB300) and the issue-bound FP32 kernels.
+// the current GPU: the FP64 rate that the FP64 kernels work around (two FMAs per
+// SM and clock on a GB300) and the ceiling of the issue-bound FP32 kernels.
 //
 // Every thread runs independent FMA chains (enough of them to cover the
 // pipelines' latency) for a fixed trip count on a grid of several resident

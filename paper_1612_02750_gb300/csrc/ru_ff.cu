@@ -2,12 +2,12 @@
 //
 // A mixed-precision solve recomputes its residual r = b - A x from the FP64
 // solution and the FP64 links every time the iterated residual has dropped
-// by delta (reliable update).  In FP64 arithmetic the two Dslash passes of an
-// update are bound by the GPU's FP64 rate (two FMAs per SM and clock: 288
-// FMAs a site take about 2.6 times as long as the pass's HBM traffic).  The
-// updates that cannot end the solve run here instead: every real is carried
-// as an unevaluated sum hi + lo of two FP32 numbers (about 47 significant
-// bits), on the FP32 pipes.
+// by delta (reliable update).  On request the updates that cannot end the solve
+// run here instead of in FP64: every real is carried as an unevaluated sum
+// hi + lo of two FP32 numbers (about 47 significant bits), on the FP32 pipes, at
+// about 165 us a pass on 32^4.  That was faster than FP64 while the GPU's FP64
+// rate bounded the FP64 passes (252 us); with their hops on the integer pipe they
+// take 131 us, and FP64 is the faster choice as well as the default.
 //
 // * FP64 inputs are split as they are loaded, with integer instructions: hi
 //   takes the leading 24 bits of the significand (truncated), lo the next 23;
