@@ -200,17 +200,10 @@ def measured_peak():
 
 
 def kernel_source_hash() -> str:
-    """Hash of the Dslash kernel's device code: the shared headers and the
-    kernel section of dslash.cu (host-side launch code excluded)."""
-    h = hashlib.sha256()
-    for rel in ("paper_1612_02750_gb300/csrc/qex_common.cuh", "paper_1612_02750_gb300/csrc/qex_dslash_site.cuh"):
-        with open(os.path.join(ROOT, rel), "rb") as f:
-            h.update(f.read())
-    with open(os.path.join(ROOT, "paper_1612_02750_gb300/csrc/dslash.cu"), "rb") as f:
-        src = f.read()
-    a, b = src.find(b"struct DsParams"), src.find(b"// Shape of a Dslash launch")
-    h.update(src[a:b] if 0 <= a < b else src)
-    return h.hexdigest()[:16]
+    """Hash of the Dslash kernel's code: the shared headers and dslash.cu."""
+    csrc = "paper_1612_02750_gb300/csrc/"
+    return files_hash([csrc + f for f in ("qex_common.cuh", "qex_dslash_site.cuh", "qex_dslash_params.cuh",
+                                          "dslash.cu")])
 
 
 def files_hash(rels) -> str:
