@@ -134,15 +134,15 @@ static int split_grid(const qex_lattice *lat, int epi, bool reduces, int per_sm)
 }
 
 template <>
-void launch_split<double>(const qex_lattice *lat, int, bool naik, int epi, const DsParams<double> &P, cudaStream_t st) {
-    launch_split_n<double, 0>(split_grid(lat, epi, P.S != nullptr, kSplitMinBlocks64), lat->pdl != 0, naik, epi, P,
-                              st);
+void launch_split<double>(const qex_lattice *lat, int, bool naik, int epi, const DsParams<double> &P, bool pdl,
+                          cudaStream_t st) {
+    launch_split_n<double, 0>(split_grid(lat, epi, P.S != nullptr, kSplitMinBlocks64), pdl, naik, epi, P, st);
 }
 
 template <>
-void launch_split<float>(const qex_lattice *lat, int fmt, bool naik, int epi, const DsParams<float> &P, cudaStream_t st) {
+void launch_split<float>(const qex_lattice *lat, int fmt, bool naik, int epi, const DsParams<float> &P, bool pdl,
+                         cudaStream_t st) {
     const int grid = split_grid(lat, epi, P.S != nullptr, kSplitMinBlocks32);
-    const bool pdl = lat->pdl != 0;
     if (fmt == 0)
         launch_split_n<float, 0>(grid, pdl, naik, epi, P, st);
     else if (fmt == 1)

@@ -138,5 +138,6 @@ extern "C" qex_status qex_normal_op_static(const qex_lattice *lat, qex_prec prec
     a.epi = EPI_NORMAL;
     a.q = in;
     a.m2 = mass * mass;
+    a.chained = !capturing(s);  // as qex_normal_op
     return launch_dslash(l, a, s);
 }

@@ -68,6 +68,7 @@ inline int64_t split_limit(bool fp64, int fmt, bool naik) {
     return naik ? 230000 : 52000;
 }
 template <typename R>
-void launch_split(const qex_lattice *lat, int fmt, bool naik, int epi, const DsParams<R> &P, cudaStream_t st);
+void launch_split(const qex_lattice *lat, int fmt, bool naik, int epi, const DsParams<R> &P, bool pdl,
+                  cudaStream_t st);
 
 }  // namespace qex

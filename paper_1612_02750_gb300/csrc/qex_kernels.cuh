@@ -138,9 +138,12 @@ struct DslashArgs {
                          // PLAIN writes nothing and RESID takes D in = 0 (r = b)
     int skip_ff;         // EPI_PLAIN / EPI_RESID of a mixed solve's update: return at once when
                          // S->ru_ff (the float-float kernels run it)
+    int chained;         // a split kernel may come up while the kernel before it, one of the same call,
+                         // still runs
 };
 
 qex_status launch_dslash(qex_lattice *lat, const DslashArgs &a, cudaStream_t st);
+bool capturing(cudaStream_t st);  // (or a stream that cannot be inspected)
 
 // ------------------------------------------------------------ multi-RHS CG
 // Per-right-hand-side CG scalars (all active right-hand sides iterate in

@@ -275,6 +275,8 @@ qex_status measure(qex_lattice *lat, qex_prec prec, const void *fat, const void 
     return QEX_OK;
 }
 
+}  // namespace
+
 bool capturing(cudaStream_t st) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
@@ -283,6 +285,8 @@ bool capturing(cudaStream_t st) {
     }
     return cs != cudaStreamCaptureStatusNone;
 }
+
+namespace {
 
 qex_status tune(qex_lattice *lat, qex_prec prec, const void *fat, const void *lng, cudaStream_t st, bool tune_blas,
                 bool force) {
