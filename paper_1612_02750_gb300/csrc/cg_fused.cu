@@ -159,6 +159,7 @@ __device__ __forceinline__ bool fused_sum(double part, double *partials, unsigne
             ok = arrive_and_wait(arrived, err, target, timeout_cycles);
         }
         ok = __shfl_sync(0xffffffffu, ok, 0);
+        __syncwarp();  // orders the lanes' reads after lane 0's acquire, which a shuffle does not
         if (ok) {
             double t = 0.0;
             for (int k = lane; k < (int)gridDim.x; k += 32) t += __ldcg(partials + k);
