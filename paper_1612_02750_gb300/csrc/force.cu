@@ -121,7 +121,8 @@ force_kernel(const __grid_constant__ Geom g, const double *__restrict__ links, d
     uint32_t mb = 0;
 #pragma unroll
     for (int c = 0; c < 3; ++c) mb = fix_max(mb, fix_max(fix_mag(e.b.c[c].re), fix_mag(e.b.c[c].im)));
-    mb = fix_range(mb, w.bad, [&] { return fix_any(e.b); });
+    bool none = false;
+    mb = fix_range(mb, w.bad, none, [&] { return fix_any(e.b); });
     uint32_t top = 0;  // leading bits of the largest |w|
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
@@ -143,8 +144,9 @@ force_kernel(const __grid_constant__ Geom g, const double *__restrict__ links, d
         wi[c] = digits_of(im);
         nr[c] = digits_of(-re);
         ni[c] = digits_of(-im);
-        br[c] = digits_of((int64_t)fix_vec_real(e.b.c[c].re, kb, false));
-        bi[c] = digits_of((int64_t)fix_vec_real(e.b.c[c].im, kb, false));
+        uint32_t lead;
+        br[c] = digits_of((int64_t)fix_vec_real(e.b.c[c].re, kb, false, lead));
+        bi[c] = digits_of((int64_t)fix_vec_real(e.b.c[c].im, kb, false, lead));
     }
     const double unit = coef * fix_double((uint64_t)(uint32_t)(unit_exp + 1023) << 52);
     Cplx<double> off[3];

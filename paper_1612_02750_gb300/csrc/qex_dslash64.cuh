@@ -55,11 +55,44 @@ struct Direction64 {
     }
 };
 
-// (D in)(x) with FP64 FMAs alone, for sites out of the fixed-point range.
+// Colour a of (D in)(x) with FP64 FMAs alone, for what fixed point does not serve.
 template <bool NAIK, typename In>
-__device__ __noinline__ Vec3<double> dslash_site_fma(const Geom &g, const double *fat, const double *lng, double c3,
-                                                     int p, int i, const In in) {
-    return dslash_site<double, 0, NAIK>(g, fat, lng, c3, p, i, site_of(g, p, i), in);
+__device__ __forceinline__ double2 dslash_colour_fma(const Geom &g, const double *fat, const double *lng, double c3,
+                                                     int p, int i, int a, const In &in) {
+    const size_t vh = (size_t)g.vh;
+    const Site s = site_of(g, p, i);
+    double2 acc = make_double2(0.0, 0.0);
+#pragma unroll 2
+    for (int h = 0; h < (NAIK ? 16 : 8); ++h) {
+        const int mu = NAIK ? h >> 2 : h >> 1, k = NAIK && (h & 2) ? 3 : 1;
+        const bool back = h & 1;
+        const int j = hop_index(g, s, mu, back ? -k : k);
+        const bool minus = ((eta_bit(s, mu) ^ (back ? bc_bit_bwd(g, s, mu, k) : bc_bit_fwd(g, s, mu, k))) != 0) != back;
+        const double2 *u = reinterpret_cast<const double2 *>(k == 1 ? fat : lng) +
+                           (size_t)((back ? 1 - p : p) * 4 + mu) * 9 * vh + (back ? j : i);
+        const Vec3<double> v = in(j);
+        double re = 0.0, im = 0.0;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const double2 e = __ldg(u + (back ? 3 * b + a : 3 * a + b) * vh);
+            const double ui = back ? -e.y : e.y;
+            re = fma(e.x, v.c[b].re, re);
+            re = fma(-ui, v.c[b].im, re);
+            im = fma(e.x, v.c[b].im, im);
+            im = fma(ui, v.c[b].re, im);
+        }
+        const double c = k == 3 ? c3 : 1.0;
+        acc.x = fma(minus ? -c : c, re, acc.x);
+        acc.y = fma(minus ? -c : c, im, acc.y);
+    }
+    return acc;
+}
+
+// ... as a call of its own, where its registers would cost the caller.
+template <bool NAIK, typename In>
+__device__ __noinline__ double2 dslash_colour_call(const Geom &g, const double *fat, const double *lng, double c3,
+                                                   int p, int i, int a, const In in) {
+    return dslash_colour_fma<NAIK>(g, fat, lng, c3, p, i, a, in);
 }
 
 // (D in)(x) for the i-th site x (= s) of parity p.  slot: the thread's words
@@ -72,7 +105,7 @@ __device__ __forceinline__ Vec3<double> dslash_site64(const Geom &g, const doubl
     Vec3<double> sum;
 #pragma unroll
     for (int a = 0; a < 3; ++a) sum.c[a].re = sum.c[a].im = 0.0;
-    bool bad = false;
+    bool bad = false, few[3] = {false, false, false};
 #pragma unroll 1
     for (int k = 1; k <= (NAIK ? 3 : 1); k += 2) {
         const double *links = !NAIK || k == 1 ? fat : lng;
@@ -130,9 +163,18 @@ __device__ __forceinline__ Vec3<double> dslash_site64(const Geom &g, const doubl
             const double re = fma(unit, (double)f.a[2 * a], t[a].re), im = fma(unit, (double)f.a[2 * a + 1], t[a].im);
             sum.c[a].re = k == 1 ? re : fma(c3, re, sum.c[a].re);
             sum.c[a].im = k == 1 ? im : fma(c3, im, sum.c[a].im);
+            few[a] |= f.some && fix_few(f.terms[a]);
         }
     }
-    if (bad) return dslash_site_fma<NAIK>(g, fat, lng, c3, p, i, in);
+    if (bad || few[0] || few[1] || few[2])
+#pragma unroll 1
+        for (int a = 0; a < 3; ++a) {
+            if (!(bad || (a == 0 ? few[0] : a == 1 ? few[1] : few[2]))) continue;
+            const double2 w = dslash_colour_fma<NAIK>(g, fat, lng, c3, p, i, a, in);
+            if (a == 0) sum.c[0] = {w.x, w.y};
+            if (a == 1) sum.c[1] = {w.x, w.y};
+            if (a == 2) sum.c[2] = {w.x, w.y};
+        }
     return sum;
 }
 

@@ -125,11 +125,16 @@ struct DirSums {
     }
 };
 
+// As kFixTerms, for sums whose alignment drops up to a unit a direction more: 20 x
+// 2^-53 of the terms' sum.
+constexpr float kDirTerms = 0x1.8p-11f;
+
 template <int FMT, bool NAIK, int SITES>
 struct DirSums<double, FMT, NAIK, SITES> {
     static constexpr int N = NAIK ? 2 : 1;
     int64_t v[N][4][6][SITES];
     int e[N][4][SITES];
+    FixMag terms[N][4][3][SITES];  // negative: the direction's hops are all zeros
     int bad[4][SITES];
 
     template <typename In>
@@ -138,45 +143,50 @@ struct DirSums<double, FMT, NAIK, SITES> {
         const size_t vh = (size_t)g.vh;
         const Site s = site_of(g, p, i);
         FixSum f;
-        f.bad = false;
+        bool out = false;
 #pragma unroll 1
         for (int n = 0; n < N; ++n) {
             const double *links = n ? lng : fat;
             const DirHop h = dir_hop(g, s, mu, 2 * n + 1);
-            f.e = 0;
-#pragma unroll
-            for (int c = 0; c < 6; ++c) f.a[c] = 0;
+            fix_clear(f);
             fix_hop<false>(f, load_link(links, vh, p, mu, i), in(h.jf), h.nf);
             fix_hop<true>(f, load_link(links, vh, 1 - p, mu, h.jb), in(h.jb), h.nb);
 #pragma unroll
             for (int c = 0; c < 6; ++c) v[n][mu][c][slot] = f.a[c];
             e[n][mu][slot] = f.e;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) terms[n][mu][c][slot] = f.some ? f.terms[c] : fix_const2(-1.f);
+            out |= f.bad;
         }
-        bad[mu][slot] = f.bad;
+        bad[mu][slot] = out;
     }
     template <typename In>
     __device__ __forceinline__ double2 get(const Geom &g, const double *fat, const double *lng, double c3, int p, int i,
                                            int a, int slot, const In &in) const {
-        if (bad[0][slot] | bad[1][slot] | bad[2][slot] | bad[3][slot]) {
-            const Vec3<double> w = dslash_site_fma<NAIK>(g, fat, lng, c3, p, i, in);
-            return a == 0 ? make_double2(w.c[0].re, w.c[0].im)
-                          : a == 1 ? make_double2(w.c[1].re, w.c[1].im) : make_double2(w.c[2].re, w.c[2].im);
-        }
+        bool redo = bad[0][slot] | bad[1][slot] | bad[2][slot] | bad[3][slot];  // fixed point does not serve
         double2 out = make_double2(0.0, 0.0);
 #pragma unroll
         for (int n = 0; n < N; ++n) {
             const int top = max(max(e[n][0][slot], e[n][1][slot]), max(e[n][2][slot], e[n][3][slot]));
             int64_t re = 0, im = 0;
+            FixMag sum = fix_const2(0.f);
+            bool some = false;
 #pragma unroll
             for (int d = 0; d < 4; ++d) {
                 const uint32_t sh = (uint32_t)(top - e[n][d][slot]);
                 re += fix_sar(v[n][d][2 * a][slot], sh);
                 im += fix_sar(v[n][d][2 * a + 1][slot], sh);
+                const FixMag t = terms[n][d][a][slot];
+                const bool none = fix_least(t) < 0.f;
+                some |= !none;
+                sum = fix_add2(sum, none ? fix_const2(0.f) : fix_lower(t, sh));
             }
+            redo |= some && fix_few(sum, kDirTerms);
             const double unit = n ? c3 * fix_unit(top) : fix_unit(top);
             out.x = fma(unit, (double)re, out.x);
             out.y = fma(unit, (double)im, out.y);
         }
+        if (redo) return dslash_colour_call<NAIK>(g, fat, lng, c3, p, i, a, in);
         return out;
     }
 };

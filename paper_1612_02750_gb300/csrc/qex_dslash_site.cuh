@@ -53,8 +53,6 @@ __device__ __forceinline__ void dslash_site_n(const Geom &g, const R *fat, const
                 for (int k = 0; k < K; ++k) {
                     if constexpr (FMT == 2)
                         acc_mv_fix16(acc[k], sg, u, in(j, k));
-                    else if constexpr (std::is_same<R, double>::value)
-                        acc_mv_unit(acc[k], sg < R(0), u, in(j, k));
                     else
                         acc_mv(acc[k], sg, u, in(j, k));
                 }
@@ -74,8 +72,6 @@ __device__ __forceinline__ void dslash_site_n(const Geom &g, const R *fat, const
                 for (int k = 0; k < K; ++k) {
                     if constexpr (FMT == 2)
                         acc_mdv_fix16(acc[k], sg, u, in(j, k));
-                    else if constexpr (std::is_same<R, double>::value)
-                        acc_mdv_unit(acc[k], sg < R(0), u, in(j, k));
                     else
                         acc_mdv(acc[k], sg, u, in(j, k));
                 }
@@ -116,7 +112,7 @@ __device__ __forceinline__ void dslash_site_n(const Geom &g, const R *fat, const
 }
 
 // One field: (D in)(x), `in(j)` the input vector at index j.  (FP64 kernels:
-// dslash_site64 in qex_dslash64.cuh, which falls back to this one.)
+// dslash_site64 in qex_dslash64.cuh.)
 template <typename R, int FMT, bool NAIK, typename In>
 __device__ __forceinline__ Vec3<R> dslash_site(const Geom &g, const R *fat, const R *lng, R c3, int p, int i,
                                                const Site &s, const In &in) {

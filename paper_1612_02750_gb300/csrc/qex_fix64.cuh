@@ -11,19 +11,35 @@
 //
 // Accuracy.  One unit of the accumulators is 2^-56 of the largest product
 // |U| |v| (largest real of the link times largest real of the vectors, each
-// rounded up to a power of two); a hop rounds by about 0.3 units, and the
-// running exponent carries kFixSlack spare bits.  FP64 arithmetic rounds
-// every partial sum by 2^-54 of its value.  Norm-wise error of a sum of eight
-// hops against 113 bits, Gaussian vectors: 0.64e-16 here, 2.3e-16 for FMAs
+// rounded up to a power of two); a hop rounds by about 0.3 units and by 2.75 at
+// most, and the running exponent carries kFixSlack spare bits.  FP64 arithmetic
+// rounds every partial sum by 2^-54 of its value.  Norm-wise error of a sum of
+// eight hops against 113 bits, Gaussian vectors: 0.64e-16 here, 2.3e-16 for FMAs
 // (unit links: 0.71e-16 and 1.05e-16; vectors of very different size from
-// hop to hop: 0.88e-16 and 2.2e-16).  The accuracy is that of the colour
-// vector as a whole: a colour far below the others of its own site keeps
-// their absolute error.  A hop whose link or vector holds an Inf or NaN, or
-// whose largest real lies outside 2^-470 .. 2^470 (zeros apart), makes the
-// site fall back to FP64 FMAs, so such values come out as they do there.
+// hop to hop: 0.88e-16 and 2.2e-16).
+//
+// That is against the largest product of the site.  A real whose own terms are all
+// far smaller (a colour, or imaginary parts, decades below the others, in links
+// that do not mix them) would lose bits that FMAs keep.  So each hop also adds up,
+// in packed halves and a little above its truth, what the magnitudes of every
+// real's terms come to, and a colour with a real whose terms do not reach kFixTerms
+// is formed again with FMAs.  The rest are within 18 x 2^-53 of their terms' sum, where
+// the 48 FMAs they stand for are within 48, and rms at 0.1 to 0.9 of those.
+// Gaussian vectors meet no such site (1e-4 of them with Gaussian links); where
+// every site is one (unit links, or colours 1e-2 apart with links that do not mix
+// them) the operator takes 330-385 us at 32^4 in place of 141.  The halves' 40
+// instructions a hop cost 8 % (byte magnitudes through __dp4a: 40 %, it takes as
+// long as an FP64 FMA).
+//
+// A hop whose link or vector holds an Inf or NaN, or whose largest real lies
+// outside 2^-470 .. 2^470 (zeros apart), makes the site fall back to FP64 FMAs as
+// well, so such values come out as they do there.
 #pragma once
 
+#include <math.h>
 #include <string.h>
+
+#include <cuda_fp16.h>
 
 #include "qex_common.cuh"
 
@@ -33,6 +49,7 @@ constexpr int kFixShift = 4;   // high digits are at most 2^28
 constexpr int kFixSlack = 1;   // spare bits of the running exponent
 constexpr int kFixLow = 553;    // exponent fields accepted: 2^-470 <= ...
 constexpr int kFixHigh = 1493;  // ... < 2^470
+constexpr float kFixTerms = 0x1p-11f;  // what FixSum::terms has to come to: 2^54 units, 2^53 at least in truth
 
 struct Digits {
     int hi, lo;  // hi 2^32 + lo
@@ -100,13 +117,95 @@ QEX_HD Digits fix_digits(uint32_t hi, uint32_t lo) {
     return d;
 }
 
+// Magnitudes of a complex value by the leading 12 bits n of its high digits, read
+// as the bits of two halves: n 2^-24 up to n = 2^11, at most twice that above.
+#ifdef __CUDA_ARCH__
+typedef __half2 FixMag;
+#else
+struct FixMag {
+    float x, y;
+};
+inline float fix_half(uint32_t n) {
+    return n < 0x400 ? ldexpf((float)n, -24) : ldexpf((float)((n & 0x3FF) | 0x400), (int)(n >> 10) - 25);
+}
+#endif
+
+QEX_HD FixMag fix_mag2(uint32_t re, uint32_t im) {
+#ifdef __CUDA_ARCH__
+    const uint32_t w = __byte_perm(re, im, 0x7632);
+    FixMag m;
+    memcpy(&m, &w, 4);
+    return m;
+#else
+    return {fix_half(re >> 16), fix_half(im >> 16)};
+#endif
+}
+
+QEX_HD FixMag fix_const2(float x) {
+#ifdef __CUDA_ARCH__
+    return __float2half2_rn(x);
+#else
+    return {x, x};
+#endif
+}
+
+QEX_HD FixMag fix_min2(FixMag a, FixMag b) {
+#ifdef __CUDA_ARCH__
+    return __hmin2(a, b);
+#else
+    return {a.x < b.x ? a.x : b.x, a.y < b.y ? a.y : b.y};
+#endif
+}
+
+QEX_HD FixMag fix_mul2(FixMag a, FixMag b) {
+#ifdef __CUDA_ARCH__
+    return __hmul2(a, b);
+#else
+    return {a.x * b.x, a.y * b.y};
+#endif
+}
+
+QEX_HD FixMag fix_swap2(FixMag a) {
+#ifdef __CUDA_ARCH__
+    return __lowhigh2highlow(a);
+#else
+    return {a.y, a.x};
+#endif
+}
+
+// c + (a.x + i a.y's magnitudes)(b.x + i b.y's): re and im; bx: b swapped.
+QEX_HD FixMag fix_terms2(FixMag a, FixMag b, FixMag bx, FixMag c) {
+#ifdef __CUDA_ARCH__
+    return __hfma2(__high2half2(a), bx, __hfma2(__low2half2(a), b, c));
+#else
+    return {a.x * b.x + a.y * bx.x + c.x, a.x * b.y + a.y * bx.y + c.y};
+#endif
+}
+
+QEX_HD FixMag fix_add2(FixMag a, FixMag b) {
+#ifdef __CUDA_ARCH__
+    return __hadd2(a, b);
+#else
+    return {a.x + b.x, a.y + b.y};
+#endif
+}
+
+QEX_HD float fix_least(FixMag a) {
+#ifdef __CUDA_ARCH__
+    return fminf(__low2float(a), __high2float(a));
+#else
+    return a.x < a.y ? a.x : a.y;
+#endif
+}
+
 // Link real: a negative one is complemented instead of negated (one unit of
 // 2^-60 off), a zero of either sign stays 0.
-QEX_HD Digits fix_link_real(double d, uint32_t key) {
+QEX_HD Digits fix_link_real(double d, uint32_t key, uint32_t &lead) {
     const uint64_t b = fix_bits(d);
     const uint32_t h = (uint32_t)(b >> 32);
     const uint64_t x = fix_abs(h, (uint32_t)b, key);
     uint32_t hi = (uint32_t)(x >> 32), lo = (uint32_t)x;
+    lead = hi;
     if (h > 0x80000000u) {
         hi = ~hi;
         lo = ~lo;
@@ -115,10 +214,11 @@ QEX_HD Digits fix_link_real(double d, uint32_t key) {
 }
 
 // Vector real times (neg ? -1 : 1), exactly negated.
-QEX_HD uint64_t fix_vec_real(double d, uint32_t key, bool neg) {
+QEX_HD uint64_t fix_vec_real(double d, uint32_t key, bool neg, uint32_t &lead) {
     const uint64_t b = fix_bits(d);
     const uint32_t h = (uint32_t)(b >> 32);
     const uint64_t x = fix_abs(h, (uint32_t)b, key);
+    lead = (uint32_t)(x >> 32);
     return ((int32_t)h < 0) != neg ? 0 - x : x;
 }
 
@@ -128,25 +228,45 @@ constexpr int kFixUnit = 2 * 1023 + 2 * (63 - kFixShift) - 64;
 struct FixSum {
     int64_t a[6];
     int e;
+    FixMag terms[3];  // what the terms of colour a come to, re and im, in units of 2^65: within [0.9, 2] of the truth
+    bool some;        // a hop was not all zeros
     bool bad;
 };
+
+// terms 2^-n (nothing left past 14)
+QEX_HD FixMag fix_lower(FixMag t, uint32_t n) {
+#ifdef __CUDA_ARCH__
+    const uint32_t w = n < 15u ? (15u - n) * 0x04000400u : 0u;
+    FixMag p;
+    memcpy(&p, &w, 4);
+    return __hmul2(t, p);
+#else
+    const float p = n < 15u ? ldexpf(1.f, -(int)n) : 0.f;
+    return {t.x * p, t.y * p};
+#endif
+}
+
+QEX_HD bool fix_few(FixMag terms, float least = kFixTerms) { return fix_least(terms) < least; }
 
 QEX_HD void fix_clear(FixSum &s) {
     for (int k = 0; k < 6; ++k) s.a[k] = 0;
     s.e = 0;
+    for (int a = 0; a < 3; ++a) s.terms[a] = fix_const2(0.f);
+    s.some = false;
     s.bad = false;
 }
 
 QEX_HD uint32_t fix_max(uint32_t a, uint32_t b) { return a > b ? a : b; }
 
 // The largest magnitude m (high word) of a link or vector, raised to the
-// smallest accepted one if all of it is zero (any() is the OR of its words);
-// bad is set if it is out of range.
+// smallest accepted one if all of it is zero (any() is the OR of its words),
+// which sets zero; bad is set if it is out of range.
 template <typename Any>
-QEX_HD uint32_t fix_range(uint32_t m, bool &bad, const Any &any) {
+QEX_HD uint32_t fix_range(uint32_t m, bool &bad, bool &zero, const Any &any) {
     if (m >= (uint32_t)kFixHigh << 20) bad = true;
     if (m < (uint32_t)kFixLow << 20) {
         if (any() << 1) bad = true;  // a sign bit alone is a zero
+        zero = true;
         m = (uint32_t)kFixLow << 20;
     }
     return m;
@@ -171,26 +291,33 @@ QEX_HD void fix_hop(FixSum &s, const Mat3<double> &u, const Vec3<double> &v, boo
     for (int k = 0; k < 9; ++k) mu = fix_max(mu, fix_max(fix_mag(u.e[k].re), fix_mag(u.e[k].im)));
 #pragma unroll
     for (int a = 0; a < 3; ++a) mv = fix_max(mv, fix_max(fix_mag(v.c[a].re), fix_mag(v.c[a].im)));
-    mu = fix_range(mu, s.bad, [&] {
+    bool zero = false;
+    mu = fix_range(mu, s.bad, zero, [&] {
         uint64_t any = 0;
 #pragma unroll
         for (int k = 0; k < 9; ++k) any |= fix_bits(u.e[k].re) | fix_bits(u.e[k].im);
         return any;
     });
-    mv = fix_range(mv, s.bad, [&] { return fix_any(v); });
+    mv = fix_range(mv, s.bad, zero, [&] { return fix_any(v); });
     const int eu = (int)(mu >> 20), eh = eu + (int)(mv >> 20);
     if (eh > s.e) {  // a larger product than the unit allows for: raise the unit
         const int e = eh + SLACK;
 #pragma unroll
         for (int k = 0; k < 6; ++k) s.a[k] = fix_sar(s.a[k], (uint32_t)(e - s.e));
+#pragma unroll
+        for (int a = 0; a < 3; ++a) s.terms[a] = fix_lower(s.terms[a], (uint32_t)(e - s.e));
         s.e = e;
     }
     const uint32_t ku = ((uint32_t)(eu + kFixShift) << 20) | 0xFFFFFu;
     const uint32_t kv = ((uint32_t)(s.e - eu + kFixShift) << 20) | 0xFFFFFu;
     Digits vr[3], vi[3], vn[3];  // vn: -vi (DAG: -vr)
+    FixMag vm[3], vx[3];         // |vr|, |vi| times 2^15 (at most 4: exact), and swapped
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-        const uint64_t re = fix_vec_real(v.c[b].re, kv, neg), im = fix_vec_real(v.c[b].im, kv, neg);
+        uint32_t lr, li;
+        const uint64_t re = fix_vec_real(v.c[b].re, kv, neg, lr), im = fix_vec_real(v.c[b].im, kv, neg, li);
+        vm[b] = fix_mul2(fix_min2(fix_mag2(lr, li), fix_const2(0x1p-13f)), fix_const2(0x1p15f));
+        vx[b] = fix_swap2(vm[b]);
         vr[b] = fix_digits((uint32_t)(re >> 32), (uint32_t)re);
         vi[b] = fix_digits((uint32_t)(im >> 32), (uint32_t)im);
         const uint64_t n = 0 - (DAG ? re : im);
@@ -204,7 +331,9 @@ QEX_HD void fix_hop(FixSum &s, const Mat3<double> &u, const Vec3<double> &v, boo
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
             const int k = DAG ? 3 * b + a : 3 * a + b;
-            const Digits ur = fix_link_real(u.e[k].re, ku), ui = fix_link_real(u.e[k].im, ku);
+            uint32_t lr, li;
+            const Digits ur = fix_link_real(u.e[k].re, ku, lr), ui = fix_link_real(u.e[k].im, ku, li);
+            s.terms[a] = fix_terms2(fix_mag2(lr, li), vm[b], vx[b], s.terms[a]);
             // U: (ur vr - ui vi, ur vi + ui vr);  U^+: (ur vr + ui vi, ur vi - ui vr)
             const Digits x = DAG ? vi[b] : vn[b], y = DAG ? vn[b] : vr[b];
             hr = fix_mad(ur.hi, vr[b].hi, hr);
@@ -223,6 +352,7 @@ QEX_HD void fix_hop(FixSum &s, const Mat3<double> &u, const Vec3<double> &v, boo
         s.a[2 * a] = fix_mad((int)(mr >> 32), 1, hr);
         s.a[2 * a + 1] = fix_mad((int)(mi >> 32), 1, hi);
     }
+    s.some |= !zero;
 }
 
 // The unit of a sum as a double (a power of two in range for a sum that is
