@@ -16,13 +16,18 @@
 namespace qex {
 
 // G has rank one, so U G = (U a) b^+ with a the vector at the hop's end and b
-// the one at x.  2 TA(U G) is then a mat-vec and 30 real products (72 FP64
-// operations a link; forming G and multiplying it by U took about 200).  They
-// run in fixed point on the integer pipe (qex_fix64.cuh), which leaves 18 FP64
-// operations, the conversions of the nine results: the FP64 pipe bounded the
-// kernel (24^4 with long links, 916 us; 32^4, 1.45 ms); now it is HBM (115 us of
-// traffic at 24^4) and the integer issue: 158 us, 288 us.  Links out of the
-// fixed-point range take FP64 FMAs.
+// the one at x.  2 TA(U G) is then a mat-vec, w = U a, and 30 real products (72 FP64
+// operations a link; forming G and multiplying it by U took about 200, 916 us on
+// 24^4 with long links).  All of it runs on the integer pipe (qex_fix64.cuh), where a
+// link takes about 1400 instructions, and leaves nothing to the FP64 pipe, whose
+// instructions cost 64 clocks each and hardly overlap with the integer ones: 224 us
+// against 115 us of HBM traffic.  w is summed under one exponent, like the
+// operator's hops, and where a real of it has only terms far below the largest the
+// link takes FP64 FMAs.  The products of w and b would meet such reals too often
+// (sums of four products, not of 36), so there every real has its own exponent,
+// and a sum takes the largest of its four.  With w and b under one exponent each it
+// took 165 us but lost the small reals; the products as FP64 FMAs 266 us, 328 with
+// w converted to FP64 by the FP64 pipe.
 
 // The vectors a and b of link (x, mu) and the sign of its G.
 struct ForceEnds {
@@ -90,100 +95,112 @@ __device__ __noinline__ void force_fma(const Geom &g, const double *links, doubl
     store_force(o, vh, off, d);
 }
 
-__device__ __forceinline__ Digits digits_of(int64_t x) {
-    return fix_digits((uint32_t)((uint64_t)x >> 32), (uint32_t)x);
+// +-a b summed over n products, their units brought to the largest's; F's elements.
+struct ForceSum {
+    int64_t x;
+    int e;  // as fix_to_double's
+};
+
+__device__ __forceinline__ int force_exp(int a, int b) { return a > b ? a : b; }
+
+// p0 + p1 - p2 - p3, p_k = a_k b_k.
+__device__ __forceinline__ ForceSum force_sum4(const FixNum &a0, const FixNum &b0, const FixNum &a1, const FixNum &b1,
+                                               const FixNum &a2, const FixNum &b2, const FixNum &a3,
+                                               const FixNum &b3) {
+    const int e0 = a0.e + b0.e, e1 = a1.e + b1.e, e2 = a2.e + b2.e, e3 = a3.e + b3.e;
+    const int e = force_exp(force_exp(e0, e1), force_exp(e2, e3));
+    return {fix_product(a0, b0, e - e0) + fix_product(a1, b1, e - e1) - fix_product(a2, b2, e - e2) -
+                fix_product(a3, b3, e - e3),
+            e};
 }
 
-// x y added to h 2^32 + m (units of digit products hi lo), as in fix_hop.
-__device__ __forceinline__ void add_product(int64_t &h, int64_t &m, const Digits &x, const Digits &y) {
-    h = fix_mad(x.hi, y.hi, h);
-    m = fix_mad(x.hi, y.lo, m);
-    m = fix_mad(x.lo, y.hi, m);
+// Its unit, 2^(e - 2 kFixNum + 64), as fix_to_double takes it.
+__device__ __forceinline__ double force_double(int64_t x, int e) {
+    return fix_to_double(x, e - 2 * kFixNum + 64 + kFixUnit);
 }
 
-// 128 threads, 6 blocks an SM (85 registers): 24^4 with long links 158 us, 162 at
-// 5 blocks (96 registers), 182 at 2 blocks of 256.
-constexpr int kForceBlock = 128;
-constexpr int kForceUnit = kFixUnit + (1023 + 63 - kFixShift) - 64;  // exponent bias of the products' unit
+// 64 threads, 10 blocks an SM (96 registers): 224 us, as 128 x 5; 264 with 256 x 2
+// (a link that takes FMAs holds its block up).
+constexpr int kForceBlock = 64;
+// What the terms of w's reals have to come to (fix_few), lower than the operator's
+// kFixTerms: the roundings of one hop, not of six, stand against them (15 x 2^-53 of
+// the terms' sum at most).
+constexpr float kForceTerms = 0x1.8p-14f;
 
-__global__ void __launch_bounds__(kForceBlock, 6)
+__global__ void __launch_bounds__(kForceBlock, 10)
 force_kernel(const __grid_constant__ Geom g, const double *__restrict__ links, double coef, int hop,
              const double *__restrict__ X, const double *__restrict__ Y, double *__restrict__ out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.vh) return;
     const size_t vh = (size_t)g.vh;
-    const ForceEnds e = force_ends(g, hop, X, Y, i);
+    ForceEnds e = force_ends(g, hop, X, Y, i);
     const Mat3<double> u = load_link(links, vh, blockIdx.y >> 2, blockIdx.y & 3, i);
     double2 *o = reinterpret_cast<double2 *>(out) + (size_t)blockIdx.y * 9 * vh + i;
-    FixSum w;  // U a
-    fix_clear(w);
-    fix_hop<false, 0>(w, u, e.a, e.neg);
-    uint32_t mb = 0;
+    FixSum f;  // U a
+    fix_clear(f);
+    fix_hop<false, 0>(f, u, e.a, e.neg);
+    if (coef != 1.0) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) mb = fix_max(mb, fix_max(fix_mag(e.b.c[c].re), fix_mag(e.b.c[c].im)));
-    bool none = false;
-    mb = fix_range(mb, w.bad, none, [&] { return fix_any(e.b); });
-    uint32_t top = 0;  // leading bits of the largest |w|
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const int h = (int)(w.a[k] >> 32);
-        top |= (uint32_t)(h ^ (h >> 31));
+        for (int c = 0; c < 3; ++c) {
+            e.b.c[c].re *= coef;
+            e.b.c[c].im *= coef;
+        }
     }
-    const int up = __clz((int)top) - kFixShift;  // 1 to 28: w's largest high digit to 27 or 28 bits
-    const int eb = (int)(mb >> 20), unit_exp = w.e - up + eb - kForceUnit;
-    if (w.bad || unit_exp < -900 || unit_exp > 900) {
+    uint32_t most = 0, least = ~0u;  // of b's magnitudes (zeros apart), a low word that is all there is as 1
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const double d = r ? e.b.c[c].im : e.b.c[c].re;
+            const uint32_t m = fix_mag(d) | ((uint32_t)fix_bits(d) != 0);
+            most = fix_max(most, m);
+            least = m - 1 < least ? m - 1 : least;
+        }
+    }
+    // Inf and NaN, and products that may leave the normal range: w's reals reach from
+    // 2^(unit) to 2^(unit + 62), the smallest unit of a product is 2^-60 of it
+    const int unit = f.e - kFixUnit;
+    const bool in_range = most < 0x7FF00000u && unit + (int)(most >> 20) < 1900 &&
+                          (least == ~0u || unit + (int)(least >> 20) > 60);
+    const bool few = f.some && (fix_few(f.terms[0], kForceTerms) || fix_few(f.terms[1], kForceTerms) ||
+                                fix_few(f.terms[2], kForceTerms));
+    if (f.bad || few || !in_range) {
         force_fma(g, links, coef, hop, X, Y, o, i);
         return;
     }
-    const uint32_t kb = ((uint32_t)(eb + kFixShift) << 20) | 0xFFFFFu;
-    Digits wr[3], wi[3], nr[3], ni[3], br[3], bi[3];  // w, -w, b
+    FixNum wr[3], wi[3], br[3], bi[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const int64_t re = (int64_t)((uint64_t)w.a[2 * c] << up), im = (int64_t)((uint64_t)w.a[2 * c + 1] << up);
-        wr[c] = digits_of(re);
-        wi[c] = digits_of(im);
-        nr[c] = digits_of(-re);
-        ni[c] = digits_of(-im);
-        uint32_t lead;
-        br[c] = digits_of((int64_t)fix_vec_real(e.b.c[c].re, kb, false, lead));
-        bi[c] = digits_of((int64_t)fix_vec_real(e.b.c[c].im, kb, false, lead));
+        wr[c] = fix_num(f.a[2 * c], f.e);
+        wi[c] = fix_num(f.a[2 * c + 1], f.e);
+        br[c] = fix_num(e.b.c[c].re);
+        bi[c] = fix_num(e.b.c[c].im);
     }
-    const double unit = coef * fix_double((uint64_t)(uint32_t)(unit_exp + 1023) << 52);
-    Cplx<double> off[3];
-    int64_t di[3];
+    Cplx<double> off[3], d[3];
+    int de = 2 * kFixNone;
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
-        int64_t h = 0, m = 0x80000000ll;
-        add_product(h, m, wi[r], br[r]);
-        add_product(h, m, nr[r], bi[r]);
-        di[r] = fix_mad((int)(m >> 32), 1, h);
+        de = force_exp(de, force_exp(wi[r].e + br[r].e, wr[r].e + bi[r].e));
 #pragma unroll
         for (int c = r + 1; c < 3; ++c) {
-            h = 0;
-            m = 0x80000000ll;
-            add_product(h, m, wr[r], br[c]);
-            add_product(h, m, wi[r], bi[c]);
-            add_product(h, m, nr[c], br[r]);
-            add_product(h, m, ni[c], bi[r]);
-            off[r + c - 1].re = unit * (double)fix_mad((int)(m >> 32), 1, h);
-            h = 0;
-            m = 0x80000000ll;
-            add_product(h, m, wi[r], br[c]);
-            add_product(h, m, nr[r], bi[c]);
-            add_product(h, m, nr[c], bi[r]);
-            add_product(h, m, wi[c], br[r]);
-            off[r + c - 1].im = unit * (double)fix_mad((int)(m >> 32), 1, h);
+            const ForceSum re = force_sum4(wr[r], br[c], wi[r], bi[c], wr[c], br[r], wi[c], bi[r]);
+            const ForceSum im = force_sum4(wi[r], br[c], wi[c], br[r], wr[r], bi[c], wr[c], bi[r]);
+            off[r + c - 1].re = force_double(re.x, re.e);
+            off[r + c - 1].im = force_double(im.x, im.e);
         }
     }
+    int64_t di[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+        di[r] = fix_product(wi[r], br[r], de - (wi[r].e + br[r].e)) -
+                fix_product(wr[r], bi[r], de - (wr[r].e + bi[r].e));
     const int64_t tr = di[0] + di[1] + di[2];
-    // 2 (d_r - tr / 3) = 2/3 (3 d_r - tr), with 2/3 to twice its precision
-    const double third2 = unit * (2.0 / 3.0), rest = unit * (0x1p-53 / 3.0);
-    Cplx<double> d[3];
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
+        // 2 (d_r - tr / 3) = 2/3 (3 d_r - tr), |3 d_r - tr| < 2^60: a third of 4 times it
+        const int64_t t = 3 * di[r] - tr;
         d[r].re = 0.0;
-        const double t = (double)(3 * di[r] - tr);
-        d[r].im = fma(third2, t, rest * t);
+        d[r].im = force_double(__mul64hi(t * 4, 0x5555555555555556ll), de - 1);
     }
     store_force(o, vh, off, d);
 }
@@ -244,8 +261,9 @@ extern "C" qex_status qex_force(const qex_lattice *lat, const void *fat64, const
         const int hop = set ? 3 : 1;
         double *out = (double *)(set ? out_lng : out_fat);
         if (kind == 0)
-            force_kernel<<<dim3(blocks_for(lat->vh, kForceBlock), 8), kForceBlock, 0, s>>>(lat->geom, (const double *)(set ? lng64 : fat64), coef, hop,
-                                                 (const double *)x_even, (const double *)y_odd, out);
+            force_kernel<<<dim3(blocks_for(lat->vh, kForceBlock), 8), kForceBlock, 0, s>>>(
+                lat->geom, (const double *)(set ? lng64 : fat64), coef, hop, (const double *)x_even,
+                (const double *)y_odd, out);
         else
             force_gradient_kernel<<<grid, kBlock, 0, s>>>(lat->geom, coef, hop, (const double *)x_even,
                                                           (const double *)y_odd, out);

@@ -27,7 +27,7 @@
 // the 48 FMAs they stand for are within 48, and rms at 0.1 to 0.9 of those.
 // Gaussian vectors meet no such site (1e-4 of them with Gaussian links); where
 // every site is one (unit links, or colours 1e-2 apart with links that do not mix
-// them) the operator takes 330-385 us at 32^4 in place of 141.  The halves' 40
+// them) the operator takes 330-430 us at 32^4 in place of 141.  The halves' 40
 // instructions a hop cost 8 % (byte magnitudes through __dp4a: 40 %, it takes as
 // long as an FP64 FMA).
 //
@@ -62,6 +62,16 @@ QEX_HD uint64_t fix_shr(uint64_t x, uint32_t n) {
     return r;
 #else
     return n > 63 ? 0 : x >> n;
+#endif
+}
+
+QEX_HD uint64_t fix_shl(uint64_t x, uint32_t n) {
+#ifdef __CUDA_ARCH__
+    uint64_t r;
+    asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));  // 0 for n > 63
+    return r;
+#else
+    return n > 63 ? 0 : x << n;
 #endif
 }
 
@@ -358,5 +368,56 @@ QEX_HD void fix_hop(FixSum &s, const Mat3<double> &u, const Vec3<double> &v, boo
 // The unit of a sum as a double (a power of two in range for a sum that is
 // not bad: exponent fields 2 kFixLow .. 2 kFixHigh + kFixSlack).
 QEX_HD double fix_unit(int e) { return fix_double((uint64_t)(uint32_t)(e - kFixUnit + 1023) << 52); }
+
+// ---------------------------------------------- reals with an exponent each
+// hi 2^32 + lo, 2^59 to 2^60 in magnitude, times 2^(e - kFixNum); zero: kFixNone.
+constexpr int kFixNum = 1023 + 63 - kFixShift;
+constexpr int kFixNone = -1000000;
+struct FixNum {
+    Digits d;
+    int e;
+};
+
+QEX_HD FixNum fix_num(double d) {  // d normal or zero
+    const uint64_t b = fix_bits(d);
+    const uint32_t h = (uint32_t)(b >> 32), f = (h >> 20) & 0x7FFu;
+    const uint64_t x = f ? (((b << 11) | 0x8000000000000000ull) >> kFixShift) : 0;
+    const uint64_t y = (int32_t)h < 0 ? 0 - x : x;
+    return {fix_digits((uint32_t)(y >> 32), (uint32_t)y), f ? (int)f : kFixNone};
+}
+
+QEX_HD int fix_clz(uint64_t x) {
+#ifdef __CUDA_ARCH__
+    return __clzll((long long)x);
+#else
+    return x ? __builtin_clzll(x) : 64;
+#endif
+}
+
+QEX_HD FixNum fix_num(int64_t x, int e) {  // x 2^(e - kFixUnit), |x| < 2^62
+    const int n = fix_clz((uint64_t)(x ^ (x >> 63)));
+    const int64_t y = (int64_t)fix_shl((uint64_t)x, (uint32_t)(n - 1)) >> (kFixShift - 1);
+    return {fix_digits((uint32_t)((uint64_t)y >> 32), (uint32_t)y),
+            x ? e - kFixUnit + kFixNum + kFixShift - n : kFixNone};
+}
+
+// a b / 2^64 in units of 2^(a.e + b.e - 2 kFixNum + 64), within 0.75; shifted down n.
+QEX_HD int64_t fix_product(const FixNum &a, const FixNum &b, int n) {
+    int64_t m = fix_mad(a.d.hi, b.d.lo, 0x80000000ll);
+    m = fix_mad(a.d.lo, b.d.hi, m);
+    return fix_sar(fix_mad((int)(m >> 32), 1, fix_mad(a.d.hi, b.d.hi, 0)), (uint32_t)n);
+}
+
+// x 2^(e - kFixUnit) as a double, rounded to the nearest (half away from zero), for
+// results in the normal range: about 46 clocks, where a conversion and a product
+// with the unit take 128 on the FP64 pipe.
+QEX_HD double fix_to_double(int64_t x, int e) {
+    const uint64_t mag = x < 0 ? 0 - (uint64_t)x : (uint64_t)x;
+    const int n = fix_clz(mag);
+    const uint64_t top = fix_shl(mag, (uint32_t)n);  // leading bit at 63
+    const uint64_t r = (top >> 11) + ((top >> 10) & 1);
+    const uint64_t d = r + ((uint64_t)(uint32_t)(e - kFixUnit + 63 - n + 1022) << 52);  // a carry raises the exponent
+    return fix_double(mag ? d | ((uint64_t)x & 0x8000000000000000ull) : 0);
+}
 
 }  // namespace qex

@@ -1,11 +1,14 @@
-"""Every real of the FP64 operator keeps FP64 accuracy against its own terms,
-however small it is beside the others of its site: colours and real and
+"""Every real of the FP64 operator and force keeps FP64 accuracy against its own
+terms, however small it is beside the others of its site: colours and real and
 imaginary parts that lie decades apart, in links that mix them and in links
 that do not.
 
-The bound is that of FP64 arithmetic, with u = 2^-53 and S the sum of the
+The bounds are those of FP64 arithmetic, with u = 2^-53 and S the sum of the
 magnitudes of a real's terms: 48 products (96 with long links) summed one after
-another round by at most 48 u S (96 u S)."""
+another round by at most 48 u S (96 u S).  A force real has 6 roundings in
+w = U a, 4 in its products and 6 in the trace and its third: 16 u S.  In fixed
+point w may be off by 2.75 units of 1.5 x 2^50 to its S, 15 u S, and what follows
+by 6 u S: 21 u S."""
 
 import numpy as np
 import pytest
@@ -145,3 +148,31 @@ def test_dslash_components(q, oracle_mod, naik, links, kind, s):
         for out in (q.qex_dslash(lat, "f64", fat, lng, C3, p, x), q.qex_dslash_mrhs(lat, "f64", fat, lng, C3, p, 1, x)):
             got = q.qex_unpack_field(lat, "f64", p, out).cpu().numpy()[at]
             compare(got, plain, val[at], mag[at], 96 if naik else 48)
+
+
+@pytest.mark.parametrize("links,kind,s", CASES)
+def test_force_components(q, oracle_mod, links, kind, s):
+    rng = np.random.default_rng(22)
+    u = links_of(links, rng)
+    z = spread(rng.standard_normal(fg.lattice_shape(DIMS) + (3, 2)).view(complex)[..., 0], kind, s)
+    even = fg.even_mask(DIMS)
+    x, y = np.where(even[..., None], z, 0), np.where(even[..., None], 0, z)
+    plain = oracle_mod.force(DIMS, u, x, y, None, 0.0, 0)[0]
+    lat = q.Lattice(DIMS)
+    g, _ = q.qex_force(lat, q.qex_pack_links(lat, "f64", dev(u)), None, 0.0, q.qex_pack_field(lat, "f64", 0, dev(x)),
+                       q.qex_pack_field(lat, "f64", 1, dev(y)))
+    got = q.qex_unpack_links(lat, "f64", g).cpu().numpy()
+    here = parts(z)
+    b = tuple(t[..., None, :] for t in here)
+    for mu in range(4):
+        s_mu = (signs(mu, 1) * np.where(even, 1.0, -1.0))[..., None]
+        (wr, wi), (nr, ni) = mat_vec(parts(u[..., mu, :, :]), tuple(np.roll(t, -1, axis=3 - mu) for t in here))
+        wr, wi, nr, ni = ((s_mu * t)[..., None] for t in (wr, wi, nr, ni))
+        m = wr * b[0] + wi * b[1], wi * b[0] - wr * b[1]
+        n = abs(nr * b[0]) + abs(ni * b[1]), abs(ni * b[0]) + abs(nr * b[1])
+        val = [m[0] - np.swapaxes(m[0], -1, -2), m[1] + np.swapaxes(m[1], -1, -2)]
+        mag = [n[0] + np.swapaxes(n[0], -1, -2), n[1] + np.swapaxes(n[1], -1, -2)]
+        for t in (val[1], mag[1]):
+            t -= (t[..., 0, 0] + t[..., 1, 1] + t[..., 2, 2])[..., None, None] / LD(3) * np.eye(3) * (
+                1 if t is val[1] else -1)
+        compare(got[..., mu, :, :], plain[..., mu, :, :], np.stack(val, -1), np.stack(mag, -1), 21)
