@@ -513,7 +513,8 @@ qex_status qex_cg_host(const qex_lattice *lat, qex_prec inner, const double *hos
  * cache keyed by (SM count, extents, boundary, prec, Naik) and, if the
  * environment variable QEX_TUNE_CACHE names a file, appends it there.
  * fat (and lng) are the link sets in prec's layout (read only).  The call
- * synchronises the stream.  Errors: QEX_ERR_ARG (null fat, or the stream is
+ * synchronises the stream.  On a small lattice, whose Dslash has one shape (see
+ * qex_tune_set), only the vector update is timed.  Errors: QEX_ERR_ARG (null fat, or the stream is
  * being captured), QEX_ERR_ALIGN, QEX_ERR_SHAPE (Naik with an extent < 4),
  * QEX_ERR_CUDA.
  * qex_dslash, qex_normal_op and qex_cg tune the Dslash shapes (not the

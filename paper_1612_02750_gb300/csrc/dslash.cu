@@ -181,7 +181,7 @@ static void launch_t(qex_lattice *lat, const DslashArgs &a, cudaStream_t st) {
     P.skip_ff = a.skip_ff;
     P.partials = lat->partials;
     P.counter = lat->counter;
-    if (lat->vh <= split_limit(std::is_same<R, double>::value, FMT, NAIK)) {
+    if (runs_split(lat, a.prec, NAIK)) {
         launch_split<R>(lat, FMT, NAIK, EPI, P, lat->pdl || a.chained, st);
         return;
     }

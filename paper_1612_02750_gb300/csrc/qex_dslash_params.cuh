@@ -67,6 +67,10 @@ inline int64_t split_limit(bool fp64, int fmt, bool naik) {
     if (fmt == 1) return naik ? 600000 : 42000;
     return naik ? 230000 : 52000;
 }
+inline bool runs_split(const qex_lattice *lat, qex_prec prec, bool naik) {
+    const int fmt = prec == QEX_F32_R12 ? 1 : prec == QEX_F32_R12H ? 2 : prec == QEX_F32_S16 ? 3 : 0;
+    return lat->vh <= split_limit(prec == QEX_F64, fmt, naik);
+}
 template <typename R>
 void launch_split(const qex_lattice *lat, int fmt, bool naik, int epi, const DsParams<R> &P, bool pdl,
                   cudaStream_t st);

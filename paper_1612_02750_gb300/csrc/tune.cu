@@ -6,7 +6,8 @@
 // and the grid are free at launch time.  The best shape depends on the volume
 // (a small lattice wants small blocks to reach more SMs; the reducing
 // variants want a persistent grid whose per-block reduction tail is paid once)
-// and is measured, not guessed: for one (precision, Naik) of a lattice the
+// and is measured, not guessed (for a lattice whose Dslash is the split one,
+// dslash_split.cu, which has one shape, the vector update alone): for one (precision, Naik) of a lattice the
 // tuner times, with CUDA events on scratch fields,
 //   * the plain Dslash with 256, 128 and 64 threads per block, each with one
 //     thread per site and with the grid capped at two resident waves (when
@@ -31,7 +32,7 @@
 #include <mutex>
 #include <string>
 
-#include "qex_kernels.cuh"
+#include "qex_dslash_params.cuh"
 
 namespace qex {
 
@@ -141,6 +142,21 @@ qex_status time_us(F launch, cudaStream_t st, float *us) {
 qex_status measure(qex_lattice *lat, qex_prec prec, const void *fat, const void *lng, cudaStream_t st,
                    bool tune_blas, TuneRecord *out) {
     const int naik = lng ? 1 : 0;
+    const int minb = prec == QEX_F64 ? kDslashMinBlocksF64 : kDslashMinBlocks;
+    const int def_per_sm = QEX_REDUCE_BLOCKS_PER_SM >= 0 ? QEX_REDUCE_BLOCKS_PER_SM : minb;
+    TuneRecord best;
+    memset(&best, 0, sizeof(best));
+    best.shape.ds_block = kDslashBlock;
+    best.shape.red_block = kDslashBlock;
+    best.shape.red_per_sm = def_per_sm;
+    // the Dslash of a small lattice has one shape: the compiled default stands for
+    // it, and there is nothing to time
+    const bool one_shape = runs_split(lat, prec, naik != 0);
+    if (one_shape && !tune_blas) {
+        lat->shape[prec][naik] = best.shape;
+        *out = best;
+        return QEX_OK;
+    }
     const size_t fb = (size_t)lat->vh * (prec == QEX_F64 ? 48 : 24);
     char *f = nullptr;
     CgScalars *S = nullptr;
@@ -162,21 +178,13 @@ qex_status measure(qex_lattice *lat, qex_prec prec, const void *fat, const void 
     LaunchShape &cur = lat->shape[prec][naik];
     const LaunchShape saved = cur;
     const int saved_blas = lat->blas_per_sm;
-    const int minb = prec == QEX_F64 ? kDslashMinBlocksF64 : kDslashMinBlocks;
-    const int def_per_sm = QEX_REDUCE_BLOCKS_PER_SM >= 0 ? QEX_REDUCE_BLOCKS_PER_SM : minb;
-    TuneRecord best;
-    memset(&best, 0, sizeof(best));
-    best.shape.ds_block = kDslashBlock;
-    best.shape.red_block = kDslashBlock;
-    best.shape.red_per_sm = def_per_sm;
-
     DslashArgs a = {};
     a.prec = prec;
     a.fat = fat;
     a.lng = lng;
     a.c3 = lng ? -1.0 / 24.0 : 0.0;
     a.m2 = 0.01;
-    do {
+    if (!one_shape) do {
         // plain Dslash: block size, one thread per site or two resident waves
         a.epi = EPI_PLAIN;
         a.out_parity = 1;
@@ -238,13 +246,15 @@ qex_status measure(qex_lattice *lat, qex_prec prec, const void *fat, const void 
                 best.shape.red_per_sm = cand[k][1];
             }
         }
-        if (s) break;
+    } while (0);
+    if (!s) {
         cur = best.shape;
         if (tune_blas) {
             // the CG vector update in prec, in the form the solve runs: FP64
             // x += alpha p, r -= alpha A p, ||r||^2; FP32 without the iterate
             // (the mixed solve folds it into the next iteration's Dslash)
             void *const xu = prec == QEX_F64 ? f0 : nullptr;
+            float t_best = 0.f;
             const int caps[4] = {QEX_BLAS_BLOCKS_PER_SM > 0 ? QEX_BLAS_BLOCKS_PER_SM : 4, 2, 8, 16};
             void *pb[2] = {f2, f2};
             const GraphCtl off = {};
@@ -260,7 +270,7 @@ qex_status measure(qex_lattice *lat, qex_prec prec, const void *fat, const void 
                 }
             }
         }
-    } while (0);
+    }
     cudaStreamSynchronize(st);
     cudaFree(f);
     cudaFree(S);
