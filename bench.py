@@ -21,6 +21,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -199,26 +200,49 @@ def measured_peak():
         return FALLBACK_HBM_GBS, "fallback"
 
 
+DSLASH_FILES = ["paper_1612_02750_gb300/csrc/" + f for f in (
+    "qex_common.cuh", "qex_kernels.cuh", "qex_dslash_site.cuh", "qex_dslash_params.cuh", "dslash.cu")]
+
+
+def device_code(src: str) -> str:
+    """The device code of a CUDA source: types, constants and macros, and the
+    functions with a __global__, __device__ or QEX_HD in front of them, without
+    comments and with single spaces.  The host's functions are left out."""
+    src = re.sub(r"//[^\n]*|/\*.*?\*/", " ", src, flags=re.S)
+    src = re.sub(r"^[ \t]*#[ \t]*(include|pragma once).*$", " ", src, flags=re.M)
+    src = re.sub(r'\b(namespace\s*\w*|extern\s*"C")\s*\{', " ", src)  # their closing braces stay behind
+    out, depth, start = [], 0, 0
+    for k, c in enumerate(src):
+        depth = max(0, depth + (c == "{") - (c == "}"))
+        if depth or c not in ";}":
+            continue
+        head = src[start:k + 1].split("{", 1)[0]
+        if c == "}" and "(" not in head and head.strip() != "}":
+            continue  # a type or a table: it goes on to its semicolon
+        if "(" not in head or re.search(r"__global__|__device__|QEX_HD|#", head):
+            out.append(src[start:k + 1])
+        start = k + 1
+    return re.sub(r"\s+", " ", " ".join(out)).strip()
+
+
 def kernel_source_hash() -> str:
-    """Hash of the Dslash kernel's code: the shared headers and dslash.cu."""
-    csrc = "paper_1612_02750_gb300/csrc/"
-    return files_hash([csrc + f for f in ("qex_common.cuh", "qex_dslash_site.cuh", "qex_dslash_params.cuh",
-                                          "dslash.cu")])
+    """Hash of the FP32 Dslash kernel's device code."""
+    return files_hash(DSLASH_FILES)
 
 
 def files_hash(rels) -> str:
-    """Hash of whole source files (kernels outside dslash.cu)."""
+    """Hash of the device code of source files."""
     h = hashlib.sha256()
     for rel in rels:
-        with open(os.path.join(ROOT, rel), "rb") as f:
-            h.update(f.read())
+        with open(os.path.join(ROOT, rel), encoding="utf-8") as f:
+            h.update(device_code(f.read()).encode())
     return h.hexdigest()[:16]
 
 
 def ncu_traffic(kernel_key: str):
     """DRAM bytes per launch from the committed ncu summary, or None when the
-    kernel source changed since the capture (the Dslash device code, or the
-    files a record names in "hash_files")."""
+    kernel changed since the capture (the FP32 Dslash's device code, or that of
+    the files a record names in "hash_files")."""
     path = os.path.join(ROOT, "profiles", "roofline_traffic.json")
     try:
         with open(path) as f:
