@@ -5,7 +5,7 @@
 //   1. p_new = r + beta p_old formed on the fly at every neighbour read,
 //      tmp = D_oe p_new, and p_new stored (two p buffers, chosen by the parity
 //      of the device-side iteration count; FP64 CG forms p_new in a separate
-//      pass, because its Dslash is FP64-ALU bound);
+//      pass: its Dslash is bound by instruction issue);
 //   2. A p_new = m^2 p_new - D_eo tmp with <p_new, A p_new> -> alpha;
 //   3. x += alpha p_new, r -= alpha A p_new, ||r||^2 -> beta or a halt flag.
 // In a mixed solve the iterate update of kernel 3 moves into the next
@@ -165,8 +165,8 @@ static qex_status enqueue_iteration(Solve &s, const GraphCtl &ctl, cudaStream_t 
             x = nullptr;
         }
     } else {
-        // FP64: the Dslash is FP64-ALU bound, so the update is its own
-        // memory-bound pass instead of eight recomputations per site
+        // FP64: the Dslash is bound by instruction issue, so the update is its
+        // own memory-bound pass instead of eight recomputations per site
         if ((err = launch_update_p(lat, a.prec, r, pb, S, st))) return err;
         if ((err = mark(marks, k++, st))) return err;
         a.epi = EPI_PLAIN;

@@ -487,7 +487,6 @@ batch_norm2_kernel(const LatDesc *__restrict__ descs, int n, BatchScalars *S, do
     __shared__ double smem[32];
     __shared__ double tot[kMaxRhs];
     __shared__ int ident[kMaxRhs + 1];
-    extern __shared__ double2 stage[];
     const int l = lattice_of_full_tile(descs, n, blockIdx.x);
     const LatDesc &D = descs[l];
     const size_t vh = (size_t)D.g.vh;

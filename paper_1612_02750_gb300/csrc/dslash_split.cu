@@ -107,7 +107,8 @@ dslash_split_kernel(const __grid_constant__ DsParams<R> P) {
 
 template <typename R, int FMT, bool NAIK>
 static void launch_split_t(int grid, bool pdl, int epi, const DsParams<R> &P, cudaStream_t st) {
-    auto kernel = epi == EPI_PLAIN ? dslash_split_kernel<R, FMT, NAIK, EPI_PLAIN> : dslash_split_kernel<R, FMT, NAIK, EPI_NORMAL>;
+    auto kernel = epi == EPI_PLAIN ? dslash_split_kernel<R, FMT, NAIK, EPI_PLAIN>
+                                   : dslash_split_kernel<R, FMT, NAIK, EPI_NORMAL>;
     if constexpr (std::is_same<R, double>::value) {
         if (epi == EPI_RESID) kernel = dslash_split_kernel<R, FMT, NAIK, EPI_RESID>;
     } else {
