@@ -105,7 +105,8 @@ __device__ __forceinline__ Vec3<double> dslash_site64(const Geom &g, const doubl
     Vec3<double> sum;
 #pragma unroll
     for (int a = 0; a < 3; ++a) sum.c[a].re = sum.c[a].im = 0.0;
-    bool bad = false, few[3] = {false, false, false};
+    bool bad = false, few[3] = {false, false, false}, ample[3];
+    int e1 = 0;
 #pragma unroll 1
     for (int k = 1; k <= (NAIK ? 3 : 1); k += 2) {
         const double *links = !NAIK || k == 1 ? fat : lng;
@@ -158,11 +159,16 @@ __device__ __forceinline__ Vec3<double> dslash_site64(const Geom &g, const doubl
         }
         bad |= f.bad;
         const double unit = fix_unit(f.e);
+        if (k == 1) e1 = f.e;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const double re = fma(unit, (double)f.a[2 * a], t[a].re), im = fma(unit, (double)f.a[2 * a + 1], t[a].im);
             sum.c[a].re = k == 1 ? re : fma(c3, re, sum.c[a].re);
             sum.c[a].im = k == 1 ? im : fma(c3, im, sum.c[a].im);
+            if (k == 1)
+                ample[a] = f.some && !fix_few(f.terms[a], 2.f * kFixTerms);
+            else if (ample[a] && fix_below(c3, f.e, e1))
+                continue;  // the one-hop terms alone serve for both
             few[a] |= f.some && fix_few(f.terms[a]);
         }
     }

@@ -164,6 +164,8 @@ struct DirSums<double, FMT, NAIK, SITES> {
     __device__ __forceinline__ double2 get(const Geom &g, const double *fat, const double *lng, double c3, int p, int i,
                                            int a, int slot, const In &in) const {
         bool redo = bad[0][slot] | bad[1][slot] | bad[2][slot] | bad[3][slot];  // fixed point does not serve
+        bool ample = false;  // the one-hop terms serve for the three-hop ones as well
+        int top1 = 0;
         double2 out = make_double2(0.0, 0.0);
 #pragma unroll
         for (int n = 0; n < N; ++n) {
@@ -181,7 +183,11 @@ struct DirSums<double, FMT, NAIK, SITES> {
                 some |= !none;
                 sum = fix_add2(sum, none ? fix_const2(0.f) : fix_lower(t, sh));
             }
-            redo |= some && fix_few(sum, kDirTerms);
+            if (n == 0) {
+                ample = some && !fix_few(sum, 2.f * kDirTerms);
+                top1 = top;
+            }
+            redo |= some && fix_few(sum, kDirTerms) && !(n == 1 && ample && fix_below(c3, top, top1));
             const double unit = n ? c3 * fix_unit(top) : fix_unit(top);
             out.x = fma(unit, (double)re, out.x);
             out.y = fma(unit, (double)im, out.y);

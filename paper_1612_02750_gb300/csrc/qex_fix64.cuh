@@ -258,6 +258,10 @@ QEX_HD FixMag fix_lower(FixMag t, uint32_t n) {
 
 QEX_HD bool fix_few(FixMag terms, float least = kFixTerms) { return fix_least(terms) < least; }
 
+// |c| 2^e <= 2^f: a sum in units of c 2^e loses no more than one in units of 2^f.  With
+// terms of twice kFixTerms in the second they are enough for both.
+QEX_HD bool fix_below(double c, int e, int f) { return (int)(fix_mag(c) >> 20) - 1022 + e <= f; }
+
 QEX_HD void fix_clear(FixSum &s) {
     for (int k = 0; k < 6; ++k) s.a[k] = 0;
     s.e = 0;
