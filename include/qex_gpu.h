@@ -92,7 +92,14 @@ typedef enum {
  * Long (Naik) links have the format qex_long_links_prec(prec): QEX_F64 and
  * QEX_F32 keep their own; QEX_F32_R12 uses QEX_F32 (long links are not
  * unitary, so two-row storage does not apply); QEX_F32_R12H and QEX_F32_S16
- * use QEX_F32_S16. */
+ * use QEX_F32_S16.
+ * The QEX_F64 operators and the force give every real to the accuracy of FP64
+ * FMAs relative to its own terms: within 48 x 2^-53 of the sum of their
+ * magnitudes (96 x 2^-53 with long links), however small it is beside the other
+ * reals of its site.  Most products run in 60-bit fixed point; sites that this
+ * would not serve (components decades apart that the links do not mix, unit
+ * links, values beyond 2^-470 .. 2^470, Inf, NaN) take FP64 FMAs, which is up to
+ * three times slower where all sites are such. */
 typedef enum { QEX_F64 = 0, QEX_F32 = 1, QEX_F32_R12 = 2, QEX_F32_R12H = 3, QEX_F32_S16 = 4 } qex_prec;
 
 typedef struct qex_lattice qex_lattice; /* opaque, owned by the library */

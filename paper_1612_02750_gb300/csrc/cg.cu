@@ -48,8 +48,8 @@ static size_t align256(size_t n) { return (n + 255) & ~size_t(255); }
 // default (cg_fused.cu).  Fused / graph, us an iteration: 16-bit 16^3 x 32
 // 22.8/23.4, 20^4 25.7/25.7; with Naik 16^4 20.6/24.9, 16^3 x 32 29.9/29.4; FP32 and
 // two-row FP32 20^4 27.7/30.9 and 25.5/26.9; with Naik 24^4 81/83 and 72/74;
-// FP64 8^4 13.6/22.5, 16^4 37.5/40.1, 16^3 x 32 66.0/61.7; with Naik 12^4 33.4/35.0,
-// 16^4 62.5/62.0.
+// FP64 8^4 10.6/19.8, 16^4 38.3/38.9, 16^3 x 24 52.8/50.4; with Naik 12^4 35.9/35.3,
+// 14^4 38.5/41.7, 16^4 68.2/64.2.
 static int64_t fused_max_vh(qex_prec inner, bool naik) {
     if (inner == QEX_F64) return naik ? 16384 : 32768;
     if (inner == QEX_F32_R12H || inner == QEX_F32_S16) return naik ? 32768 : 65536;

@@ -335,8 +335,8 @@ qex_status qex_normal_op(const qex_lattice *lat, qex_prec prec, const void *fat,
     a.epi = EPI_NORMAL;
     a.q = in;
     a.m2 = mass * mass;
-    // a small lattice's second kernel comes up while the first runs (8^4, FP64: 8.2 us
-    // a call, 12.3 before); under capture the kernels stay plain nodes
+    // a small lattice's second kernel comes up while the first runs (8^4, FP64: 9.0 us
+    // a call, about 4 more without); under capture the kernels stay plain nodes
     a.chained = !capturing(s);
     return launch_dslash(l, a, s);
 }

@@ -7,7 +7,7 @@
 // block is 32 sites by four warps, warp mu takes the two (four) hops along mu,
 // all of whose loads are in flight at once, and the sums meet in shared memory,
 // from which three of the warps run the epilogue, one colour each.  8^4 FP64:
-// 9.0 -> 3.3 us (Naik 18.3 -> 5.3), 16-bit 3.0 -> 1.9 us; where it ends:
+// 10.0 -> 3.4 us (Naik 20.9 -> 5.8), 16-bit 3.0 -> 1.9 us; where it ends:
 // split_limit.
 #include "qex_dslash_params.cuh"
 #include "qex_dslash_dir.cuh"

@@ -19,7 +19,7 @@ namespace qex {
 // the one at x.  2 TA(U G) is then a mat-vec, w = U a, and 30 real products (72 FP64
 // operations a link; forming G and multiplying it by U took about 200, 916 us on
 // 24^4 with long links).  All of it runs on the integer pipe (qex_fix64.cuh), where a
-// link takes about 1400 instructions, and leaves nothing to the FP64 pipe, whose
+// link takes about 1800 instructions, and leaves nothing to the FP64 pipe, whose
 // instructions cost 64 clocks each and hardly overlap with the integer ones: 224 us
 // against 115 us of HBM traffic.  w is summed under one exponent, like the
 // operator's hops, and where a real of it has only terms far below the largest the

@@ -3,17 +3,20 @@
 // FP64 FMAs alone need 288 x 64 clocks a warp and SM quarter (32^4: 250 us,
 // the FP64 pipe's limit, against 96 us of HBM traffic).  Here the x, y and z
 // hops run in fixed point on the integer pipe (qex_fix64.cuh: 72 % of the
-// work, about 1070 clocks a warp and hop) and the t hops as FP64 FMAs that are
-// issued between them, so both pipes work at once: 131 us at 32^4 (617 against
-// 1264 at 48^4; with the Naik term 257 against 502).  All hops on the integer
-// pipe: 136 us; the t hops as a part of their own after or before the others:
-// 135-136 us.  What bounds it now is the integer issue (two clocks an
-// instruction, about 3400 a site) next to the HBM traffic.
+// work, about 1180 clocks a warp and hop) and the t hops as FP64 FMAs that are
+// issued between them, so both pipes work at once: 141 us at 32^4 (651 against
+// 1264 at 48^4; with the Naik term 288-304 against 502).  Before the hops kept the
+// bound on their terms it was 131 us; at that time, all hops on the integer pipe took
+// 136 us, the t hops as a part of their own after or before the others 135-136 us.
+// What bounds it now is the integer issue (two clocks an instruction, 4750 a site)
+// next to the HBM traffic.
 //
 // The t hops' links and vectors wait in shared memory (cp.async, 384 bytes a
 // thread, read back by the thread that copied them, so no barrier): loaded
 // where they are used they cost 160 us, in registers they spill.  128
-// registers, 16 warps an SM; 96 registers and 20 warps spill (140-165 us).
+// registers, 16 warps an SM; 96 registers and 20 warps spilt (140-165 us).  Without
+// the Naik term 20 to 40 bytes spill, with it 180 to 310, in L1.  The fallback stands
+// inline, two hops a trip: 139 us, as a call 148 to 158, fully unrolled 155.
 #pragma once
 
 #include "qex_dslash_site.cuh"

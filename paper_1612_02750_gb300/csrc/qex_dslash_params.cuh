@@ -55,8 +55,9 @@ __device__ __forceinline__ void finish_reduction(const DsParams<R> &P, double pa
 
 // Largest half volume whose Dslash splits each site's directions over four
 // threads (dslash_split.cu); fmt: the fat links' format (qex_dslash_site.cuh).
-// Split / one thread a site, us: FP64 20^4 24.6/28.9, 20 x 22^3 31.5/31.8; with
-// Naik 24^3 x 48 169/174, 32^4 264/258.  FP32 16^2 x 20^2 4.2/4.3, 16^3 x 32
+// Split / one thread a site, us: FP64 20^4 25.8/31.1, 20 x 22^3 33.4/34.6, 24^4
+// 50.4/49.4; with Naik 24^3 x 48 184/196, 32^4 288/304, 36^4 471/459 (the line lies
+// lower: they were 264/258 at 32^4 before the hops kept their bound).  FP32 16^2 x 20^2 4.2/4.3, 16^3 x 32
 // 5.0/4.6; with Naik 24^3 x 32 40.8/41.2, 28^4 54.5/51.4.  Two-row FP32 16^4
 // 3.4/3.6, 16^2 x 20^2 4.3/4.1; with Naik 32^4 72.8/76.2, 40^4 183/189 (at HBM
 // both).  16-bit 10 x 14 x 18 x 22 3.3/3.4, 16^4 3.6/3.4; with Naik 16^4

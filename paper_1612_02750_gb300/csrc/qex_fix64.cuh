@@ -3,11 +3,11 @@
 // An FP64 FMA takes 64 clocks a warp on a GB300 SM quarter, a 32x32+64-bit
 // integer multiply-add and every other integer instruction 2 (measured; the
 // two kinds of integer instruction share those clocks).  A 3x3 complex
-// mat-vec is 36 FP64 FMAs, 2304 clocks; here it takes 1070: the link and the
+// mat-vec is 36 FP64 FMAs, 2304 clocks; here it takes 1180: the link and the
 // vector are brought into fixed point (a common exponent each, 60 bits, as
 // two signed 32-bit digits), a product is three multiply-adds (hi hi, hi lo,
 // lo hi; the lo lo product is below the last bit kept) and the sums are exact
-// 64-bit integers.  About half of the 520 instructions convert the link.
+// 64-bit integers.  About half of the 600 instructions convert the link.
 //
 // Accuracy.  One unit of the accumulators is 2^-56 of the largest product
 // |U| |v| (largest real of the link times largest real of the vectors, each
@@ -27,7 +27,7 @@
 // the 48 FMAs they stand for are within 48, and rms at 0.1 to 0.9 of those.
 // Gaussian vectors meet no such site (1e-4 of them with Gaussian links); where
 // every site is one (unit links, or colours 1e-2 apart with links that do not mix
-// them) the operator takes 330-430 us at 32^4 in place of 141.  The halves' 40
+// them) the operator takes 330-430 us at 32^4 in place of 141.  The bound's 80
 // instructions a hop cost 8 % (byte magnitudes through __dp4a: 40 %, it takes as
 // long as an FP64 FMA).
 //

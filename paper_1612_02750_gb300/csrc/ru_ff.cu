@@ -7,7 +7,7 @@
 // hi + lo of two FP32 numbers (about 47 significant bits), on the FP32 pipes, at
 // about 165 us a pass on 32^4.  That was faster than FP64 while the GPU's FP64
 // rate bounded the FP64 passes (252 us); with their hops on the integer pipe they
-// take 131 us, and FP64 is the faster choice as well as the default.
+// take 141 us, and FP64 is the faster choice as well as the default.
 //
 // * FP64 inputs are split as they are loaded, with integer instructions: hi
 //   takes the leading 24 bits of the significand (truncated), lo the next 23;
